@@ -71,7 +71,7 @@ def tracer_sha():
     """Hash of the tracer kernel's sources and of the default grid cells (which set its traffic)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2501_05828_gb300", "csrc")
-    for f in ("ur_trace.cu", "ur_device.cuh"):
+    for f in ("ur_trace.cuh", "ur_trace.cu", "ur_device.cuh"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "ur_api.cu"), "rb") as fh:

@@ -384,8 +384,8 @@ ur_status ur_graph_launch(ur_ctx *ctx);
  * a plane z = c or a cylinder along y (plane waves of a linear array then never
  * gain a y component, so thin y cells add few cell steps and hold fewer
  * scatterers); 3 r_s, 3 r_s and 40 r_s when the scene holds a sphere.  block (multiple of 32, <= 256), blocks_per_sm and
- * resolve_batch (1..32: the tracer finishes segments and starts rays once this
- * many lanes of a warp wait; default 20) apply at the next trace. */
+ * resolve_batch (1..32: the tracer starts new rays once this many lanes of a warp
+ * are without one; default 10) apply at the next trace. */
 typedef struct {
     float cell_xy, cell_z;
     int32_t block, blocks_per_sm, resolve_batch;

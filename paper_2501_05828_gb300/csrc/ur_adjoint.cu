@@ -9,6 +9,7 @@
 // no derivative.  At every arrival the loss sensitivities dL/d(amplitude) and
 // dL/d(time) are formed from dL/d(rf, quad) over the pulse taps (Eq. 14) and
 // chained into the parameter gradient.
+#define UR_COMPILER_SUMS
 #include "ur_device.cuh"
 
 #include <algorithm>

@@ -76,7 +76,7 @@ constexpr float kCellIso[3] = {6.f, 6.f, 4.f};
 // scene.  83 % of the layered frame's reference tests came from such segments.
 constexpr float kCellFine[3] = {0.5f, 0.5f, 10.f};
 constexpr double kFineMaxCells = (double)(1u << 24);
-constexpr int kResolveBatch = 20;   // default: lanes that must wait before a tracer warp resolves segments
+constexpr int kResolveBatch = 10;   // default: lanes of a tracer warp without a ray before it starts new ones
 
 struct SceneData {
     bool ok = false;

@@ -23,7 +23,8 @@ constexpr int kMaxTri = 1 << 22;   // triangles per scene (hit ids stay below 2^
 constexpr int kBvhStack = 32;      // traversal stack; the host's BVH is never deeper
 constexpr int kGeoConvex = 1;      // tracer instantiation bits: convex array,
 constexpr int kGeoMesh = 2;        // triangle-mesh boundaries,
-constexpr int kGeoEmit = 4;        // synthetic-aperture transmits or transmit mixing
+constexpr int kGeoEmit = 4;      // synthetic-aperture transmits or transmit mixing,
+constexpr int kGeoOne = 8;       // launches of one scene
 constexpr uint64_t kFnvOffset = 0xcbf29ce484222325ull;
 constexpr uint64_t kFnvPrime = 0x100000001b3ull;
 
@@ -116,7 +117,27 @@ __device__ __forceinline__ uint64_t fnv_step(uint64_t h, uint32_t w) { return (h
 __device__ __forceinline__ float3 operator+(float3 a, float3 b) { return make_float3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ float3 operator-(float3 a, float3 b) { return make_float3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ float3 operator*(float s, float3 a) { return make_float3(s * a.x, s * a.y, s * a.z); }
+// Sums of products in the tracer's path geometry are written with their fused operations, in one
+// order: a ray's decisions (branches, captures, beam tests) compare such sums, so every
+// instantiation of the tracer must round them alike whatever the compiler would have fused in its
+// place.  (The adjoint evaluates a recorded path's derivatives and leaves them to the compiler.)
+#ifdef UR_COMPILER_SUMS
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return a * b + c * d; }
 __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+#else
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return fmaf(a, b, c * d); }   // a b + c d
+__device__ __forceinline__ float dot3(float3 a, float3 b) { return fmaf(a.z, b.z, sum2(a.x, b.x, a.y, b.y)); }
+#endif
+// b + s a
+__device__ __forceinline__ float3 along(float3 b, float s, float3 a) {
+    return make_float3(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y), fmaf(s, a.z, b.z));
+}
+// s a + t b
+__device__ __forceinline__ float3 blend(float s, float3 a, float t, float3 b) {
+    return make_float3(sum2(s, a.x, t, b.x), sum2(s, a.y, t, b.y), sum2(s, a.z, t, b.z));
+}
+// The same sum in the order the connection rays and some terms of the rough boundaries' weights use.
+__device__ __forceinline__ float dot3_yx(float3 a, float3 b) { return fmaf(a.z, b.z, sum2(a.y, b.y, a.x, b.x)); }
 // Unit vector by the hardware reciprocal square root (a few ulp; the tracer's directions feed
 // geometry whose error budget is set by FP32 positions, and no slow path of an IEEE divide runs).
 __device__ __forceinline__ float3 unit3(float3 a) {
@@ -201,7 +222,7 @@ struct TraceP {
     uint2 key;
     int max_b;
     float max_path;
-    int resolve_batch;              // lanes that must wait before a warp resolves segments
+    int resolve_batch;              // lanes without a ray before a warp starts new ones
     int mix_tx;                     // > 0: the rays of item 0's slots draw their transmit among items
                                     // 0 .. mix_tx - 1 (extended tracer only)
     const uint32_t *mix_list;       // with mix_tx: the ray index of each of item 0's slots (null: slot order)
@@ -223,18 +244,22 @@ struct TraceP {
 // (id n_bnd, upward rays) and the absorbing plane z = z_max (id n_bnd + 1,
 // downward rays) take part.
 // Moeller-Trumbore: distance along o + t d to the triangle (v0, e1 = v1 - v0, e2 = v2 - v0).
+// NEE: for the connection rays of rough vertices (the order of d x e2's products, see sum2).
+template <bool NEE>
 __device__ __forceinline__ bool tri_hit(float4 v0, float4 e1, float4 e2, float3 o, float3 d, float &t) {
-    const float px = d.y * e2.z - d.z * e2.y, py = d.z * e2.x - d.x * e2.z, pz = d.x * e2.y - d.y * e2.x;
-    const float det = e1.x * px + e1.y * py + e1.z * pz;
+    const float px = NEE ? sum2(-d.z, e2.y, d.y, e2.z) : sum2(d.y, e2.z, -d.z, e2.y);
+    const float py = NEE ? sum2(-d.x, e2.z, d.z, e2.x) : sum2(d.z, e2.x, -d.x, e2.z);
+    const float pz = NEE ? sum2(-d.y, e2.x, d.x, e2.y) : sum2(d.x, e2.y, -d.y, e2.x);
+    const float det = fmaf(e1.z, pz, sum2(e1.x, px, e1.y, py));
     if (det == 0.f) return false;
     const float inv = 1.f / det;
     const float sx = o.x - v0.x, sy = o.y - v0.y, sz = o.z - v0.z;
-    const float u = (sx * px + sy * py + sz * pz) * inv;
+    const float u = fmaf(sz, pz, sum2(sx, px, sy, py)) * inv;
     if (u < 0.f || u > 1.f) return false;
-    const float qx = sy * e1.z - sz * e1.y, qy = sz * e1.x - sx * e1.z, qz = sx * e1.y - sy * e1.x;
-    const float v = (d.x * qx + d.y * qy + d.z * qz) * inv;
+    const float qx = sum2(sy, e1.z, -sz, e1.y), qy = sum2(sz, e1.x, -sx, e1.z), qz = sum2(sx, e1.y, -sy, e1.x);
+    const float v = fmaf(d.z, qz, sum2(d.x, qx, d.y, qy)) * inv;
     if (v < 0.f || u + v > 1.f) return false;
-    t = (e2.x * qx + e2.y * qy + e2.z * qz) * inv;
+    t = fmaf(e2.z, qz, sum2(e2.x, qx, e2.y, qy)) * inv;
     return true;
 }
 
@@ -268,6 +293,7 @@ __device__ __forceinline__ bool box_hit(float4 lo, float4 hi, float3 o, float3 i
 }
 
 // Nearest triangle along o + t d with t in (kTmin, best): BVH walk, near child first.
+template <bool NEE>
 __device__ __forceinline__ void nearest_triangle(const SceneP &S, float3 o, float3 d, int skip, float &best,
                                                  int &hit) {
     const int3 par = make_int3(d.x == 0.f, d.y == 0.f, d.z == 0.f);
@@ -284,7 +310,7 @@ __device__ __forceinline__ void nearest_triangle(const SceneP &S, float3 o, floa
                 const float4 v0 = S.tri[3 * q];
                 const int id = S.tri_base + __float_as_int(v0.w);
                 float t;
-                if (id != skip && tri_hit(v0, S.tri[3 * q + 1], S.tri[3 * q + 2], o, d, t) && t > kTmin &&
+                if (id != skip && tri_hit<NEE>(v0, S.tri[3 * q + 1], S.tri[3 * q + 2], o, d, t) && t > kTmin &&
                     t < best) {
                     best = t;
                     hit = id;
@@ -310,7 +336,8 @@ __device__ __forceinline__ void nearest_triangle(const SceneP &S, float3 o, floa
     }
 }
 
-template <bool MESH = false>
+// CONN: called for a connection ray from a scatterer, NEE: from a rough vertex (the order of some sums, see sum2).
+template <bool MESH = false, bool CONN = false, bool NEE = false>
 __device__ __forceinline__ int nearest(const SceneP &S, float3 o, float3 d, int skip, bool terminals,
                                        float &t_out, float radius = 0.f) {
     float best = INFINITY;
@@ -327,8 +354,8 @@ __device__ __forceinline__ int nearest(const SceneP &S, float3 o, float3 d, int 
             if (p == skip) {
                 t = -2.f * b;
             } else {
-                const float3 f = oc - b * d;
-                const float disc = B.p[3] * B.p[3] - dot3(f, f);
+                const float3 f = along(oc, -b, d);
+                const float disc = fmaf(B.p[3], B.p[3], -dot3(f, f));
                 if (disc < 0.f) continue;
                 const float s = sqrtf(disc);
                 t = -b - s;
@@ -336,14 +363,14 @@ __device__ __forceinline__ int nearest(const SceneP &S, float3 o, float3 d, int 
             }
         } else {
             const float ocx = o.x - B.p[0], ocz = o.z - B.p[1];
-            const float a = d.x * d.x + d.z * d.z;
+            const float a = CONN ? sum2(d.z, d.z, d.x, d.x) : sum2(d.x, d.x, d.z, d.z);
             if (a == 0.f) continue;
-            const float b = (ocx * d.x + ocz * d.z) / a;
+            const float b = sum2(ocx, d.x, ocz, d.z) / a;
             if (p == skip) {
                 t = -2.f * b;
             } else {
-                const float fx = ocx - b * d.x, fz = ocz - b * d.z;
-                const float disc = (B.p[2] * B.p[2] - (fx * fx + fz * fz)) / a;
+                const float fx = fmaf(-b, d.x, ocx), fz = fmaf(-b, d.z, ocz);
+                const float disc = fmaf(B.p[2], B.p[2], -sum2(fx, fx, fz, fz)) / a;
                 if (disc < 0.f) continue;
                 const float s = sqrtf(disc);
                 t = -b - s;
@@ -355,13 +382,13 @@ __device__ __forceinline__ int nearest(const SceneP &S, float3 o, float3 d, int 
             hit = p;
         }
     }
-    if (MESH && S.n_tri > 0) nearest_triangle(S, o, d, skip, best, hit);
+    if (MESH && S.n_tri > 0) nearest_triangle<NEE>(S, o, d, skip, best, hit);
     if (terminals && radius > 0.f) {   // convex probe: its cylinder (id n_bnd), the escape plane z = -R (n_bnd + 2)
         const float ox = o.x, oz = o.z + radius;
-        const float a = d.x * d.x + d.z * d.z;
-        const float b = ox * d.x + oz * d.z;
+        const float a = sum2(d.x, d.x, d.z, d.z);
+        const float b = sum2(ox, d.x, oz, d.z);
         if (a > 0.f && b < 0.f) {
-            const float disc = b * b - a * ((ox - radius) * (ox + radius) + oz * oz);
+            const float disc = fmaf(b, b, -(a * sum2(ox - radius, ox + radius, oz, oz)));
             if (disc >= 0.f) {
                 const float t = (-b - sqrtf(disc)) / a;
                 if (t > kTmin && t < best) {
@@ -441,10 +468,11 @@ __device__ __forceinline__ void surface(const SceneP &S, int hit, float3 &h, flo
 __device__ __forceinline__ bool fresnel(float cos_i, float c1, float Z1, float c2, float Z2, float &r,
                                         float &cos_t) {
     const float eta = c2 / c1;
-    const float k = 1.f - eta * eta * (1.f - cos_i * cos_i);
+    const float k = fmaf(-(eta * eta), fmaf(-cos_i, cos_i, 1.f), 1.f);
     if (k < 0.f) return false;
     cos_t = sqrtf(k);
-    r = (Z2 * cos_i - Z1 * cos_t) / (Z2 * cos_i + Z1 * cos_t);
+    const float z1t = Z1 * cos_t;
+    r = fmaf(Z2, cos_i, -z1t) / fmaf(Z2, cos_i, z1t);
     return true;
 }
 
@@ -472,8 +500,8 @@ __device__ __forceinline__ float directivity(const TraceP &P, float ax, float tr
 
 // Squared length of v x n for a unit n: the part of v across n, from products that do not cancel.
 __device__ __forceinline__ float cross2(float3 v, float3 n) {
-    const float a = v.y * n.z - v.z * n.y, b = v.z * n.x - v.x * n.z, c = v.x * n.y - v.y * n.x;
-    return a * a + b * b + c * c;
+    const float a = sum2(v.y, n.z, -v.z, n.y), b = sum2(v.z, n.x, -v.x, n.z), c = sum2(v.x, n.y, -v.y, n.x);
+    return fmaf(c, c, sum2(a, a, b, b));
 }
 
 
