@@ -380,10 +380,11 @@ ur_status ur_graph_launch(ur_ctx *ctx);
 
 /* Scatterer-grid and launch tuning (0 fields keep the defaults).  Cell sizes in
  * metres along x (cell_xy), y (cell_y) and z (cell_z), applied at the next
- * ur_scene_upload.  Defaults: 8 r_s, 0.3 r_s and 60 r_s when every boundary is
- * a plane z = c or a cylinder along y (plane waves of a linear array then never
- * gain a y component, so thin y cells add few cell steps and hold fewer
- * scatterers); 3 r_s, 3 r_s and 40 r_s when the scene holds a sphere.  block (multiple of 32, <= 256), blocks_per_sm and
+ * ur_scene_upload.  Defaults at the densities of the measured phantoms: 9 r_s, 0.15 r_s and
+ * 2 r_s when every boundary is a smooth plane z = c or cylinder along y (plane waves of a
+ * linear array then never gain a y component, so thin y cells cost no visits and hold fewer
+ * scatterers); 4, 2, 2 r_s when such boundaries are rough; 14, 14, 2 r_s with spheres or
+ * triangles; wider where scatterers are sparser, narrower where they are denser.  block (multiple of 32, <= 256), blocks_per_sm and
  * resolve_batch (1..32: the tracer starts new rays once this many lanes of a warp
  * are without one; default 10) apply at the next trace. */
 typedef struct {

@@ -54,21 +54,32 @@ constexpr uint32_t kChunk = 4096;      // most arrivals per deposit work item
 constexpr uint32_t kChunkMin = 512;    // fewest (work items are sized for several deposit waves)
 
 // One uploaded scene: host copies of media and boundaries, device scatterers and grid.
-// Default scatterer-grid cell sizes (x, y, z) in units of the capture radius
-// r_s.  The tracer walks columns in x and y; z cells only index each column's
-// references by depth (a visit reads the z cells within r_s of the depths it
-// spans).  Plane waves of a linear array travel in the xz plane, and smooth
-// planes z = c and cylinders along y keep them there (their normals have no y
-// component), so in such scenes thin y columns hold few scatterers and cost no
-// steps.  Rough boundaries scatter part of the rays out of the plane (wider y
-// columns), and spheres and triangle meshes turn every ray in 3D (square
-// columns).  Measured on the layered frame (smooth: 10.6 ms at 6 x 0.3 x 4 r_s),
-// its rough-bone version (17.7 ms at 4 x 2 x 4 against 20.0 at 6 x 0.3 x 4) and
-// the paper-settings and mesh-bone acquisitions (9.1 and 23.9 ms at 6 x 6 x 4
-// against 10.9 and 26.6 at 3 x 3 x 5).
-constexpr float kCellSlab[3] = {6.f, 0.3f, 4.f};
-constexpr float kCellRough[3] = {4.f, 2.f, 4.f};
-constexpr float kCellIso[3] = {6.f, 6.f, 4.f};
+// Default scatterer-grid cell sizes (x, y, z) in units of the capture radius r_s, at the
+// scatterer density (per r_s^3 of their bounding box) they were measured at.  The tracer visits
+// columns in x and y; z cells only index each column's references by depth (a visit reads the z
+// cells within r_s of the depths it spans).  Plane waves of a linear array travel in the xz plane,
+// and smooth planes z = c and cylinders along y keep them there (their normals have no y
+// component), so in such scenes thin y columns hold few scatterers and cost no visits.  Rough
+// boundaries scatter part of the rays out of the plane (wider y columns), and spheres and triangle
+// meshes turn every ray in 3D (square columns).
+//
+// A segment costs about C / h visits per length and, per visit, the references of a column: with
+// the density rho, C / h + rho h (thin y columns: the depth a visit spans grows with h) or
+// C / h + rho h^2 (square columns), so the best h goes with rho^-1/2 and rho^-1/3.  Measured trace
+// (us) at 4, 6, 9, 14 r_s: layered frame with 50k scatterers 4378, 4023, 3837, 3750 at 0 degrees and
+// 2673, 2410, 2326, 2431 at 10; with 5k 2105, 1685, 1387, 1205; paper settings 5498, 4866, 4425, 4258
+// (20 r_s: 4505), with 2k instead of 20k scatterers 1712, 1474, 1309, 1171, 1093 and 1043 at 30;
+// mesh bone 8094, 7573, 7205, 7066 (7303).  z cells of 2 r_s instead of 4, and y columns of 0.15
+// instead of 0.3: 1 to 2 % less each.
+struct CellRule {
+    float cell[3];
+    float density;    // scatterers per r_s^3 the sizes were measured at
+    float power;      // x (and a wide y) scale with density^-power
+    float lo, hi;     // bounds of the factor
+};
+constexpr CellRule kCellSlab = {{9.f, 0.15f, 2.f}, 4.4e-3f, 0.5f, 0.4f, 8.f};
+constexpr CellRule kCellRough = {{4.f, 2.f, 2.f}, 4.4e-3f, 1.f / 3.f, 0.5f, 6.f};
+constexpr CellRule kCellIso = {{14.f, 14.f, 2.f}, 1.1e-3f, 1.f / 3.f, 0.25f, 6.f};
 // Fine columns (x, y, z in r_s) for exactly vertical segments (every 0-degree plane-wave ray until
 // it meets a tilted boundary, and every normal-incidence echo): such a segment stays in one
 // column, so narrow columns cost it no steps and hold (0.5 + 2)^2 / pi = 2x the scatterers of
@@ -89,6 +100,7 @@ struct SceneData {
     int n_scat = 0;
     float r_s = 1e-4f;
     float g_rm = 0.f;
+    float density = 0.f;                   // scatterers per r_s^3 of their bounding box
     float cell_req[3] = {0.f, 0.f, 0.f};   // cell sizes the grid was built for (before any enlargement)
     float3 g_lo{}, g_h{}, g_inv_h{};
     int3 g_dim{};
@@ -345,7 +357,11 @@ bool rough_scene(const SceneData &sd) {
 }
 
 float default_cell(const SceneData &sd, int a) {
-    return (!planar_scene(sd) ? kCellIso : rough_scene(sd) ? kCellRough : kCellSlab)[a] * sd.r_s;
+    const CellRule &rule = !planar_scene(sd) ? kCellIso : rough_scene(sd) ? kCellRough : kCellSlab;
+    float f = 1.f;
+    if (a == 0 || (a == 1 && rule.cell[1] >= 1.f))
+        f = std::min(rule.hi, std::max(rule.lo, std::pow(rule.density / std::max(sd.density, 1e-12f), rule.power)));
+    return rule.cell[a] * f * sd.r_s;
 }
 
 // Fine columns serve the plane-wave tracer's vertical segments: smooth planar scenes only (rough
@@ -397,6 +413,9 @@ void build_grid(ur_ctx *c, SceneData &sd, const float *src) {
         if (!std::isfinite(lo[a]) || !std::isfinite(hi[a])) fail(UR_ERR_INVALID_ARG, "scatterer coordinates must be finite");
     // capture box margin: r_s plus a relative and absolute slack far above FP32 rounding
     const float r_m = sd.r_s * 1.001f + 1e-7f;
+    double box = 1.0;   // bounding box in r_s, no side under the capture tube's width
+    for (int a = 0; a < 3; ++a) box *= std::max(2.0, ((double)hi[a] - (double)lo[a]) / (double)sd.r_s);
+    sd.density = (float)((double)n / box);
     float h_x = c->tune.cell_xy > 0.f ? c->tune.cell_xy : default_cell(sd, 0);
     float h_y = c->tune.cell_y > 0.f ? c->tune.cell_y : default_cell(sd, 1);
     float h_z = c->tune.cell_z > 0.f ? c->tune.cell_z : default_cell(sd, 2);
@@ -1816,10 +1835,10 @@ ur_status ur_autotune(ur_ctx *c, int scene, uint64_t n_rays, uint64_t seed, int 
         if (cur.blocks_per_sm <= 0) cur.blocks_per_sm = ur::trace_occupancy(256, false);
         float t_cur = measure(cur);
         // coordinate descent over the knobs
-        const float z_mult[] = {2.f, 3.f, 5.f, 8.f, 12.f};
-        const float xy_mult[] = {1.f, 1.5f, 2.f, 3.f, 4.f, 6.f};
-        const float y_mult[] = {0.2f, 0.3f, 0.5f, 1.f, 2.f, 3.f};
-        const int batches[] = {8, 12, 16, 20, 24};
+        const float z_mult[] = {2.f, 4.f, 8.f};
+        const float xy_mult[] = {2.f, 4.f, 6.f, 9.f, 14.f, 20.f, 30.f};
+        const float y_mult[] = {0.2f, 0.3f, 0.5f, 1.f, 2.f, 4.f, 9.f, 14.f, 20.f};
+        const int batches[] = {1, 6, 10, 14, 20};
         for (int pass = 0; pass < 2; ++pass) {
             for (float m : z_mult) {
                 ur_tuning t = cur;
