@@ -52,6 +52,13 @@ bool is_device_ptr(const void *p) {
 constexpr double kPi = 3.14159265358979323846;
 constexpr uint32_t kChunk = 4096;      // most arrivals per deposit work item
 constexpr uint32_t kChunkMin = 512;    // fewest (work items are sized for several deposit waves)
+// Rows of this many arrivals are deposited through interpolation nodes, in work items of at most
+// kNodeChunk: one row's convolution costs what about 500 arrivals cost tap by tap, its item more the
+// closer the arrivals lie in time (deposit of the layered frame, 17.7k arrivals per row: 412 us tap by
+// tap, 272 with items of 8192, 240 with 4096, 244 with 2048; 32 x 128 rows of 1.8k arrivals: 1239, 685, 690,
+// 870 us).  Calls whose rows hold fewer on average do not launch that kernel.
+constexpr uint32_t kNodeMin = 1024;
+constexpr uint32_t kNodeChunk = 4096;
 
 // One uploaded scene: host copies of media and boundaries, device scatterers and grid.
 // Default scatterer-grid cell sizes (x, y, z) in units of the capture radius r_s, at the
@@ -135,6 +142,9 @@ struct ur_ctx {
     bool tx_dirty = true;
     bool mix_tx = false;                    // ur_trace: each ray draws its transmit
     ur::MixP mix{};                         // ray order of the last mixed trace (list null: none)
+    ur::BinP nodes{};                       // the deposit's interpolation nodes for the array's pulse
+    ur::BinNodeG node_g{};
+    bool nodes_ok = false;
     DevBuf mix_list, mix_bins;
     DevBuf adj_order, adj_keys;        // arrivals of the adjoint in path-shape order, and that sort's counts
     DevBuf delay, tx_sin, tx_cos, tx_m, tx_kind, elem_xz;
@@ -929,7 +939,7 @@ void size_trace_buffers(ur_ctx *c, uint64_t cap, bool dbg) {
     c->grow(c->row_fill, sizeof(uint32_t) * n_rows);
     c->grow(c->row_off, sizeof(uint32_t) * (n_rows + 1));
     c->grow(c->work, sizeof(uint4) * (n_rows + c->arr_cap / kChunkMin + 16));
-    c->grow(c->n_work, sizeof(uint32_t));
+    c->grow(c->n_work, 2 * sizeof(uint32_t));
 }
 
 void launch_trace_kernel(ur_ctx *c, ur::TraceP &P, bool dbg, uint2 *arr_dbg) {
@@ -955,7 +965,8 @@ void launch_trace_kernel(ur_ctx *c, ur::TraceP &P, bool dbg, uint2 *arr_dbg) {
 }
 
 // Sort the arrival queue by row and deposit the pulses (asynchronous).
-void launch_binning(ur_ctx *c, float *d_rf, float *d_q) {
+// n_arr: arrivals in the queue, as far as the host knows.
+void launch_binning(ur_ctx *c, float *d_rf, float *d_q, uint64_t n_arr) {
     const uint64_t n_rows = (uint64_t)c->items.size() * c->arr.n_el;
     const size_t out_elems = (size_t)n_rows * c->arr.n_s;
     ck(cudaMemsetAsync(d_rf, 0, sizeof(float) * out_elems, c->stream), "memset rf");
@@ -985,6 +996,16 @@ void launch_binning(ur_ctx *c, float *d_rf, float *d_q) {
     B.phase_per_sample = (float)(2.0 * (double)c->arr.f0 / (double)c->arr.fs);
     B.rot32_s = (float)std::sin(kPi * 32.0 * (double)B.phase_per_sample);
     B.rot32_c = (float)std::cos(kPi * 32.0 * (double)B.phase_per_sample);
+    B.node_min = kNodeMin;
+    B.node_chunk = kNodeChunk;
+    if (!c->nodes_ok) {   // the pulse's interpolation nodes, once per array
+        c->nodes = B;
+        ur::plan_bin_nodes(c->nodes, c->node_g, s_samples);
+        c->nodes_ok = true;
+    }
+    B.n_nodes = n_arr >= n_rows * kNodeMin ? c->nodes.n_nodes : 0;
+    std::copy(c->nodes.node, c->nodes.node + ur::kBinNodes, B.node);
+    std::copy(c->nodes.node_w, c->nodes.node_w + ur::kBinNodes, B.node_w);
     ck(cudaMemsetAsync(B.row_count, 0, sizeof(uint32_t) * n_rows, c->stream), "memset rows");
     ck(cudaMemsetAsync(B.row_fill, 0, sizeof(uint32_t) * n_rows, c->stream), "memset rows");
     c->phase_begin(UR_PHASE_SORT);
@@ -992,9 +1013,9 @@ void launch_binning(ur_ctx *c, float *d_rf, float *d_q) {
     ck(cudaGetLastError(), "sort kernels");
     c->phase_end(UR_PHASE_SORT, 3);
     c->phase_begin(UR_PHASE_DEPOSIT);
-    ur::launch_bin_deposit(B, c->sms, c->stream);
+    const int kernels = ur::launch_bin_deposit(B, c->node_g, n_rows + n_arr / kNodeChunk, c->sms, c->stream);
     ck(cudaGetLastError(), "deposit kernel");
-    c->phase_end(UR_PHASE_DEPOSIT, 1);
+    c->phase_end(UR_PHASE_DEPOSIT, kernels);
 }
 
 void read_stats(const unsigned long long *h, ur_stats *st) {
@@ -1097,7 +1118,7 @@ void do_trace(ur_ctx *c, uint64_t n_rays, uint64_t seed, int max_b, float max_pa
         c->grow(c->stage_quad, sizeof(float) * out_elems);
         d_q = (float *)c->stage_quad.p;
     }
-    launch_binning(c, d_rf, d_q);
+    launch_binning(c, d_rf, d_q, n_arr);
     if (dbg_on) {
         dbg->count = n_arr;
         ur::DebugOut D{dbg->ray, dbg->event, dbg->row, dbg->t_hi, dbg->t_lo, dbg->amp, dbg->capacity};
@@ -1321,6 +1342,7 @@ ur_status ur_set_array(ur_ctx *c, const ur_array *a) {
             fail(UR_ERR_INVALID_ARG, "radius must be 0 (linear) or a convex radius with an opening below 170 degrees");
         c->arr = A;
         c->array_ok = true;
+        c->nodes_ok = false;
         c->tx_dirty = true;
         c->batch_ok = false;
     });
@@ -1682,7 +1704,7 @@ ur_status ur_batch_trace(ur_ctx *c, uint64_t seed, int max_b, float max_path, fl
             fail(UR_ERR_STATE, "the batch plan was replaced by another trace: plan again");
         ur::TraceP P = make_trace_params(c, seed, max_b, max_path);
         launch_trace_kernel(c, P, false, nullptr);
-        launch_binning(c, rf, quad);
+        launch_binning(c, rf, quad, c->batch_cap);   // the count stays on the device
         c->prof_sync();
     });
 }

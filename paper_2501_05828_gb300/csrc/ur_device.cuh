@@ -528,6 +528,8 @@ struct AdjP {
 constexpr int kAdjKeys = 256;   // path shapes: aperture return or scatterer event x interactions before it
 void launch_adjoint(const AdjP &A, int sms, cudaStream_t s);
 
+constexpr int kBinNodes = 8;     // most interpolation nodes per cell of the deposit
+constexpr int kBinCell = 4;      // samples per cell
 struct BinP {
     const uint4 *arr;
     const unsigned long long *arr_count;
@@ -537,7 +539,7 @@ struct BinP {
     uint32_t *row_fill;     // [n_rows]
     uint32_t *row_off;      // [n_rows + 1]
     uint4 *items;           // (row, begin, end, 0) work items
-    uint32_t *n_items;
+    uint32_t *n_items;      // [2]: items deposited tap by tap (from the front of items), through nodes (from its back)
     uint32_t max_items;
     uint32_t chunk, chunk_min, target_items;   // work items of chunk_min..chunk arrivals, about target_items of them
     int priv_rows;          // row histograms in shared memory (n_rows <= kBinPrivRows)
@@ -545,11 +547,25 @@ struct BinP {
     float *rf, *quad;       // [n_rows][n_s]
     float K, inv_2s2_log2e, phase_per_sample;   // taps |n - t| <= K; log2(e) / (2 s^2); 2 f0 / fs (half-cycles per sample)
     float rot32_s, rot32_c;                     // sin, cos of the carrier phase over 32 samples
+    // rows of many arrivals: interpolation nodes (n_nodes = 0: every row is deposited tap by tap)
+    int n_nodes;
+    float node[kBinNodes], node_w[kBinNodes];   // node offsets from a cell's centre (samples), 1 / prod (x_k - x_m)
+    uint32_t node_min, node_chunk;              // rows of at least node_min arrivals, in items of node_chunk
 };
+// The pulse's Gaussian at the 4 samples of a group, by (distance of the group to a cell, node of the cell).
+constexpr int kBinDist = 64;    // most distances (pulse half-width up to about 125 samples)
+struct BinNodeG {
+    int j_lo, n_j;              // distances j_lo .. j_lo + n_j - 1 (in cells)
+    int d_lo, d_hi;             // taps (samples from the cell's centre) that every arrival of a cell has
+    float4 g[kBinDist * kBinNodes];
+};
+// Nodes per cell for a pulse of Gaussian width s and half-width K (samples): fills the BinP's node fields and G.
+void plan_bin_nodes(BinP &B, BinNodeG &G, double s);
 constexpr int kBinPrivRows = 4096;                  // largest row count with shared-memory histograms
 int bin_sort_smem(int n_rows);                      // their bytes per CTA (0: global counters)
 void launch_bin_sort(const BinP &B, int sms, cudaStream_t s);      // 3 kernels
-void launch_bin_deposit(const BinP &B, int sms, cudaStream_t s);   // 1 kernel
+// returns the kernels launched (1 or 2); most_items: bound on the node items (0: unknown)
+int launch_bin_deposit(const BinP &B, const BinNodeG &G, uint64_t most_items, int sms, cudaStream_t s);
 
 struct GridBuildP {
     const float4 *scat;
