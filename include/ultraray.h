@@ -386,7 +386,7 @@ ur_status ur_graph_launch(ur_ctx *ctx);
  * scatterers); 4, 2, 2 r_s when such boundaries are rough; 14, 14, 2 r_s with spheres or
  * triangles; wider where scatterers are sparser, narrower where they are denser.  block (multiple of 32, <= 256), blocks_per_sm and
  * resolve_batch (1..32: the tracer starts new rays once this many lanes of a warp
- * are without one; default 10) apply at the next trace. */
+ * are without one; default 18, 10 in the extended tracers) apply at the next trace. */
 typedef struct {
     float cell_xy, cell_z;
     int32_t block, blocks_per_sm, resolve_batch;

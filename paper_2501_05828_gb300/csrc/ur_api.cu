@@ -94,7 +94,7 @@ constexpr CellRule kCellIso = {{14.f, 14.f, 2.f}, 1.1e-3f, 1.f / 3.f, 0.25f, 6.f
 // scene.  83 % of the layered frame's reference tests came from such segments.
 constexpr float kCellFine[3] = {0.5f, 0.5f, 10.f};
 constexpr double kFineMaxCells = (double)(1u << 24);
-constexpr int kResolveBatch = 10;   // default: lanes of a tracer warp without a ray before it starts new ones
+constexpr int kResolveBatch = 10;   // where the autotuner starts (ur_tuning::resolve_batch)
 
 struct SceneData {
     bool ok = false;
@@ -900,7 +900,7 @@ ur::TraceP make_trace_params(ur_ctx *c, uint64_t seed, int max_b, float max_path
     P.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     P.max_b = max_b;
     P.max_path = max_path;
-    P.resolve_batch = c->tune.resolve_batch > 0 ? c->tune.resolve_batch : kResolveBatch;
+    P.resolve_batch = c->tune.resolve_batch;
     c->grow(c->counters, 8 * sizeof(unsigned long long));
     unsigned long long *cnt = (unsigned long long *)c->counters.p;
     P.arr_count = cnt;
@@ -1588,6 +1588,7 @@ ur_status ur_trace_adjoint(ur_ctx *c, uint64_t n_rays, uint64_t seed, int max_b,
         A.T = make_trace_params(c, seed, max_b, max_path);
         A.g_rf = d_g[0];
         A.g_q = d_g[1];
+        A.vec = c->arr.n_s % 4 == 0 && ((uintptr_t)d_g[0] | (uintptr_t)d_g[1]) % 16 == 0;
         c->grow(c->adj_grad, sizeof(double) * 3 * ur::kAdjMed);
         ck(cudaMemsetAsync(c->adj_grad.p, 0, sizeof(double) * 3 * ur::kAdjMed, c->stream), "memset grad");
         A.grad = (double *)c->adj_grad.p;

@@ -222,7 +222,7 @@ struct TraceP {
     uint2 key;
     int max_b;
     float max_path;
-    int resolve_batch;              // lanes without a ray before a warp starts new ones
+    int resolve_batch;              // lanes without a ray before a warp starts new ones (0: the kernel's default)
     int mix_tx;                     // > 0: the rays of item 0's slots draw their transmit among items
                                     // 0 .. mix_tx - 1 (extended tracer only)
     const uint32_t *mix_list;       // with mix_tx: the ray index of each of item 0's slots (null: slot order)
@@ -516,6 +516,7 @@ struct AdjP {
     const float *g_rf, *g_q;    // dL/d rf, dL/d quad  [n_items][n_el][n_s]
     double *grad;               // [3 * kAdjMed]: (c, Z, alpha) per medium, accumulated
     float *grad_amp;            // [n_scat] of scene 0, accumulated (nullable)
+    int vec;                    // 1: rows of g_rf and g_q start on 16 bytes
     float K, inv_2s2, inv_s2, half_cycles, om;   // pulse: half-width, 1/(2 s^2), 1/s^2 (samples), 2 f0/fs, rad/sample
     float fs, k_alpha;          // sampling frequency; d(Np/m)/d(dB/cm/MHz) at f0
     const uint4 *arr;           // arrivals of the forward trace (row, t_hi, t_lo, amp)

@@ -857,13 +857,18 @@ __device__ __forceinline__ uint32_t item_of(const TraceP &P, uint64_t slot) {
     return (uint32_t)lo;
 }
 
-// Residency: the usual tracer runs 4 CTAs per SM in 64 registers; the extended ones trade
-// warps for registers (3 CTAs, 80 registers: 14.84 instead of 15.18 ms on the paper-settings
-// acquisition, 29.6 instead of 32.0 ms on the rough layered frame), the mesh ones more so (2 CTAs, 128 registers: the BVH walk's stack and state
-// spilled 1.3 KB per thread at 64 registers; 61.5 instead of 71.5 ms).  The grid is sized for
-// 4 CTAs per SM: CTAs that find the ray pools empty exit at once.
+// Residency, trading warps for registers, measured (us) at 2, 3 and 4 CTAs per SM: plane waves in one
+// scene (constants free the registers of its fields) 3 (layered frame 3522 against 3789 at 4, one
+// 7-degree wave the same), batches of several scenes 4 (21.9 ms against 23.0 at 3), extended 3 (paper
+// settings 4773, 4200, 4910; diverging 2170, 1790, 2090), meshes 3 (mesh bone 7055, 6573, 7446).  The
+// grid is sized for 4 CTAs per SM: CTAs that find the ray pools empty exit at once.
 template <bool ROUGH, int GEO>
-constexpr int trace_ctas_per_sm() { return (GEO & kGeoMesh) ? 2 : ROUGH ? 3 : 4; }
+constexpr int trace_ctas_per_sm() { return ROUGH || (GEO & kGeoOne) ? 3 : 4; }
+
+// Lanes without a ray before a warp starts new ones.  Measured (us) at 10, 14, 18: layered frame 3532,
+// 3495, 3452, two scenes x 16 plane waves 18963, 18766, 18685; paper settings 4208, 4380, 4428, mesh bone
+// 6597, 6625, 6640 (1 and 4: layered frame 4031 and 3908 against 3761 at 10, paper settings alike).
+constexpr int kIdleMin = 18, kIdleMinExtended = 10;
 
 // Persistent tracer.  Each iteration of the warp's loop (1) takes one step of every lane's path
 // (finish the segment, start a new ray in idle lanes, set up the next segment), (2) makes the
@@ -877,13 +882,12 @@ constexpr int trace_ctas_per_sm() { return (GEO & kGeoMesh) ? 2 : ROUGH ? 3 : 4;
 //
 // Bound by instruction issue (61 % of cycles) and the latency of reference loads.  Before, each lane
 // walked its own segment, one column per iteration, and segments were finished once 20 lanes
-// waited: 425 warp instructions per ray of the layered frame with 21.7 of 32 lanes; now about 300
-// with 26.3.  Trace of the layered frame (1e7 rays, 0 degrees) 5578 -> 4020 us, the paper-settings
-// acquisition 5960 -> 4860, 9 diverging waves 3050 -> 1940, mesh bone (25 x 256k rays) 10660 -> 7560,
-// two scenes x 16 plane waves x 1e6 rays 29.3 -> 19.7 ms.  The warp synchronisations after the
-// divergent steps keep the lanes together (mesh bone 8610 -> 7760 us, paper settings 4920 -> 4630).
-// New rays start once P.resolve_batch lanes are idle: 1, 4, 10 and 14 gave 4031, 3908, 3761 and
-// 3740 us on the layered frame, and no difference where all rays of a warp end together.
+// waited: 425 warp instructions per ray of the layered frame with 21.7 of 32 lanes; this way about
+// 300 with 26.3.  Trace, in us before, with this and with the cells, residency and threshold that suit it: layered
+// frame (1e7 rays, 0 degrees) 5578, 4020, 3453; paper settings 5960, 4860, 4225; 9 diverging waves 3050,
+// 1940, 1798; mesh bone (25 x 256k rays) 10660, 7560, 6557; two scenes x 16 plane waves x 1e6 rays 29.3,
+// 19.7, 18.7 ms.  The warp synchronisations after the divergent steps keep the lanes together (mesh
+// bone 8610 -> 7760 us, paper settings 4920 -> 4630).
 template <bool DBG, bool SPLIT, bool REC, bool ROUGH, int GEO>
 __global__ void __launch_bounds__(kBlock, trace_ctas_per_sm<ROUGH, GEO>()) k_trace(const __grid_constant__ TraceP P) {
     __shared__ WarpQueue s_q[kWarps];
@@ -894,6 +898,7 @@ __global__ void __launch_bounds__(kBlock, trace_ctas_per_sm<ROUGH, GEO>()) k_tra
     ConnQueue &CQ = s_c[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const uint64_t n_slots = P.n_slots;
+    const int idle_min = P.resolve_batch > 0 ? P.resolve_batch : ROUGH ? kIdleMinExtended : kIdleMin;
     Counters cn = {0, 0, 0, 0, 0, 0};
     Lane R;
     R.state = kNeedRay;
@@ -908,7 +913,7 @@ __global__ void __launch_bounds__(kBlock, trace_ctas_per_sm<ROUGH, GEO>()) k_tra
         if (R.state == kHasSeg) finish_segment<DBG, SPLIT, REC, ROUGH, GEO>(P, R, cn);
         __syncwarp();
         unsigned need = __ballot_sync(0xffffffffu, R.state == kNeedRay);
-        if (need && (__popc(need) >= P.resolve_batch || __ballot_sync(0xffffffffu, R.state == kNeedSeg) == 0u)) {
+        if (need && (__popc(need) >= idle_min || __ballot_sync(0xffffffffu, R.state == kNeedSeg) == 0u)) {
             uint64_t my_slot = ~0ull;
             while (need) {
                 if (pool_cnt == 0) {
