@@ -357,9 +357,10 @@ __device__ __forceinline__ uint32_t start_segment(const TraceP &P, Lane &R, Coun
 // Visit k of the n of a segment o + t d (walk, box stretch [t0, t1], length seg): the references
 // `begin` .. `begin` + count of one column's z cells within g_rm of the depths its stretch spans, and
 // the stretch [t_enter, t_end) whose closest approaches it accepts.  The stretches of a segment's
-// visits share their ends (the same expression gives both), so every scatterer within r_s of the
-// segment is accepted exactly once; the first reaches g_rm before the box (no closest approach
-// lies there, the margin only keeps rounding out of play), the last to the segment's end.
+// visits share their ends (the same expression gives both) and none but the last passes t1, so every
+// scatterer within r_s of the segment is accepted exactly once; the first reaches g_rm before the
+// box and the last to the segment's end (no closest approach lies outside the box, the margins only
+// keep rounding out of play).
 template <bool FINE>
 __device__ __forceinline__ uint32_t column_visit(const SceneP &S, float3 o, float3 d, uint32_t walk, float t0, float t1,
                                                  float seg, uint32_t k, uint32_t n, uint32_t &begin,
@@ -389,7 +390,8 @@ __device__ __forceinline__ uint32_t column_visit(const SceneP &S, float3 o, floa
         const float im = __fdividef(1.f, dm);
         const auto border = [&](int b) { return (fmaf((float)b, hm, lom) - om) * im; };   // column b's lower side
         if (k > 0u) t_enter = ta = border(neg ? c + 1 : c);
-        if (k + 1u < n) t_end = tb = border(neg ? c : c + 1);
+        // for a ray that hardly crosses the columns, im magnifies the rounding of the side past the end
+        if (k + 1u < n) t_end = tb = fminf(border(neg ? c : c + 1), t1);
         const int sa = cell_at(os + ta * ds, los, inv_hs, dim_s);
         int cs = sa;
         if (dual) {
