@@ -377,6 +377,8 @@ __global__ void __launch_bounds__(kNodeThreads) k_bin_nodes(const __grid_constan
     }
 }
 
+constexpr int kNodeSmem = 226 << 10;   // most shared memory of a CTA
+
 int node_smem(const BinP &B) {
     return (2 * B.n_nodes * node_cells(B.K, B.n_s) + 2 * B.n_s) * (int)sizeof(float);
 }
@@ -384,8 +386,10 @@ int node_smem(const BinP &B) {
 template <int R>
 void launch_nodes(const BinP &B, const BinNodeG &G, uint64_t most_items, int sms, cudaStream_t s) {
     const int smem = node_smem(B);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_bin_nodes<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    uint64_t grid = (uint64_t)sms * std::max(1, std::min(4, (226 << 10) / (smem + 1024)));
+    // one value for every caller: the attribute belongs to the process, and a context of shorter rows in
+    // another thread must not lower it between this call's attribute and its launch
+    cudaFuncSetAttribute(k_bin_nodes<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNodeSmem);
+    uint64_t grid = (uint64_t)sms * std::max(1, std::min(4, kNodeSmem / (smem + 1024)));
     if (most_items) grid = std::min(grid, most_items);
     k_bin_nodes<R><<<(int)grid, kNodeThreads, smem, s>>>(B, G);
 }
@@ -468,7 +472,7 @@ void plan_bin_nodes(BinP &B, BinNodeG &G, double s) {
             B.node[k] = (float)x[k];
             B.node_w[k] = (float)w[k];
         }
-        if (node_smem(B) > (226 << 10)) {
+        if (node_smem(B) > kNodeSmem) {
             B.n_nodes = 0;
             return;
         }
