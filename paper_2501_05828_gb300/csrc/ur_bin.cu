@@ -305,10 +305,13 @@ __global__ void __launch_bounds__(kNodeThreads) k_bin_nodes(const __grid_constan
             const float re = a.z * cs, im = -a.z * sn;
             // a cell outside the row's has no taps in it (no arrival is that early or late)
             const bool use = first && n0 <= n1 && c >= 0 && c < cells;
+            // amplitudes that are not finite (or nearly overflow) would spoil every sample of their nodes:
+            // all their taps are left to the loop below
+            const bool smooth = use && fabsf(a.z) < 1e37f && dl == dl;
             // The warp adds its arrivals two at a time, half a warp per arrival and a lane per (node,
             // component): echoes of one scatterer arrive within a cell, and a lane per arrival would
             // leave the lanes of a warp waiting for one another's sums.
-            unsigned todo = __ballot_sync(0xffffffffu, use);
+            unsigned todo = __ballot_sync(0xffffffffu, smooth);
             while (todo) {
                 const int j0 = __ffs(todo) - 1;
                 todo &= todo - 1u;
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_bin_nodes(const __grid_constan
             }
             if (!use) continue;
             // taps the nodes leave out
-            const int l1 = min(n1, tc + d_lo - 1), r0 = max(n0, tc + d_hi + 1);
+            const int l1 = smooth ? min(n1, tc + d_lo - 1) : n1, r0 = max(n0, tc + d_hi + 1);
             for (int n = n0 <= l1 ? n0 : r0; n <= n1; n = n == l1 ? max(r0, l1 + 1) : n + 1) {
                 const float tau = ((float)n - a.x) - a.y;
                 const float g = a.z * exp2f(-tau * tau * B.inv_2s2_log2e);

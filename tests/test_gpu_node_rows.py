@@ -40,6 +40,26 @@ def traced(ur, w, n_rays, seed=3):
     return rf.double().cpu().numpy(), quad.double().cpu().numpy(), gpu_records(rec, w["array"]["n_el"]), launches
 
 
+def test_amplitudes_that_are_not_finite_keep_to_their_taps(ur):
+    """A scatterer whose amplitude is NaN or infinite spoils the samples its pulses cover, no others."""
+    w = workload(40e6, 1536, 5.0)
+    w["scene"]["scatterers"][7, 3] = np.nan
+    w["scene"]["scatterers"][11, 3] = np.inf
+    rf, quad, arr, launches = traced(ur, w, 200_000)
+    assert launches == 2 and np.bincount(arr["el"], minlength=4).min() >= 1024
+    bad = ~np.isfinite(arr["amp"])
+    assert 0 < bad.sum() < arr.size
+    K = 5.0 * 5.0 / (4 * w["array"]["f0"]) * w["array"]["fs"]
+    hit = np.zeros((4, 1536), bool)
+    for a in arr[bad]:
+        hit[a["el"], max(0, int(np.ceil(a["t"] - K))):int(np.floor(a["t"] + K)) + 1] = True
+    assert hit.any() and not hit.all()
+    orf, oq = oracle.deposit(w["array"], 1, arr[~bad])
+    for g, o in ((rf, orf), (quad, oq)):
+        assert np.array_equal(np.isfinite(g[0]), ~hit)
+        assert rel_l2(g[0][~hit], o[0][~hit]) <= 4e-6
+
+
 def test_simulators_of_other_row_lengths_in_other_threads(ur):
     """The node kernel's shared memory differs with the row's length; calls of several threads do not
     take one another's."""
