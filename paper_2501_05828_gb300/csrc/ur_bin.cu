@@ -244,7 +244,8 @@ __global__ void __launch_bounds__(512) k_bin_deposit(const BinP B) {
 //   rf + j quad of an arrival (t, amp) at sample n:  sin / -cos of  omega (n - t), times amp g(n - t),
 // so the row is e^(i omega n) times the sum of amp e^(-i omega t) g(n - t).  g is smooth on the scale of a
 // few samples: within a cell of 4 samples around tc, g(n - t) is its interpolation from R Chebyshev
-// nodes tc + x_k (R chosen so that the error stays below FP32's rounding of the peak), and an arrival
+// nodes tc + x_k (R chosen so that the error stays below FP32's rounding of the peak, and below that
+// of the tap itself at the pulse's weak ends, see kNodeRel), and an arrival
 // adds amp e^(-i omega t) L_k(t - tc) to its cell's R complex node sums: 2 R shared atomics instead of 2 per
 // tap (14 instead of 202).  Each sample then sums g over the nodes of the cells around it once.  Only
 // taps inside the pulse's cut |n - t| <= K for every t of a cell go through the nodes; the up to 5 others
@@ -380,6 +381,11 @@ __global__ void __launch_bounds__(kNodeThreads) k_bin_nodes(const __grid_constan
     }
 }
 
+// Interpolation error of a tap relative to its envelope.  FP32's own, tap by tap (rounded arguments of
+// the Gaussian and of the carrier), is 1e-6 RMS and 2.6e-6 to 6e-6 at most for pulses of 3 to 9 cycles at
+// 25 to 50 MHz; the bound takes 50 MHz x 5 cycles from 6 nodes (7.9e-6) to 7 (2.8e-7).
+constexpr double kNodeRel = 2.5e-6;
+
 constexpr int kNodeSmem = 226 << 10;   // most shared memory of a CTA
 
 int node_smem(const BinP &B) {
@@ -447,14 +453,15 @@ void plan_bin_nodes(BinP &B, BinNodeG &G, double s) {
     G.n_j = ((G.d_hi + kBinCell / 2) >> 2) - G.j_lo + 1;
     if (G.n_j > kBinDist) return;
     for (int R = 5; R <= kBinNodes && !B.n_nodes; ++R) {
-        double x[kBinNodes], w[kBinNodes], worst = 0.0;
+        double x[kBinNodes], w[kBinNodes], worst = 0.0, worst_rel = 0.0;
         for (int k = 0; k < R; ++k) x[k] = kBinCell / 2 * std::cos((2 * k + 1) * 3.14159265358979323846 / (2 * R));
         for (int k = 0; k < R; ++k) {
             w[k] = 1.0;
             for (int m = 0; m < R; ++m)
                 if (m != k) w[k] /= x[k] - x[m];
         }
-        // largest interpolation error of the unit-peak Gaussian over a cell and the pulse
+        // largest interpolation error of the unit-peak Gaussian over a cell and the pulse, and the largest
+        // relative to the tap itself where the nodes serve it
         for (int q = 0; q <= 32; ++q) {
             const double t = kBinCell * (q / 32.0 - 0.5);
             double L[kBinNodes];
@@ -464,12 +471,14 @@ void plan_bin_nodes(BinP &B, BinNodeG &G, double s) {
                     if (m != k) L[k] *= t - x[m];
             }
             for (int d = -(int)B.K; d <= (int)B.K; ++d) {
-                double v = -std::exp(-(d - t) * (d - t) / (2.0 * s * s));
+                const double g = std::exp(-(d - t) * (d - t) / (2.0 * s * s));
+                double v = -g;
                 for (int k = 0; k < R; ++k) v += L[k] * std::exp(-(d - x[k]) * (d - x[k]) / (2.0 * s * s));
                 worst = std::max(worst, std::fabs(v));
+                if (d >= G.d_lo && d <= G.d_hi) worst_rel = std::max(worst_rel, std::fabs(v) / g);
             }
         }
-        if (worst > 2e-8) continue;
+        if (worst > 2e-8 || worst_rel > kNodeRel) continue;
         B.n_nodes = R;
         for (int k = 0; k < R; ++k) {
             B.node[k] = (float)x[k];

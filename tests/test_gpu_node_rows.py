@@ -40,6 +40,32 @@ def traced(ur, w, n_rays, seed=3):
     return rf.double().cpu().numpy(), quad.double().cpu().numpy(), gpu_records(rec, w["array"]["n_el"]), launches
 
 
+@pytest.mark.parametrize("fs,n_cycles", [(50e6, 5.0), (40e6, 5.0), (50e6, 3.0), (25e6, 5.0), (50e6, 9.0)])
+def test_weak_ends_of_the_pulse(ur, fs, n_cycles):
+    """A plane's echo at one time, every sample relative to its own envelope (4e-6 of the peak at the cut):
+    no further off than one tap evaluated in FP32, where the carrier's argument (h half-cycles at the cut,
+    two rounded factors and their product) and the Gaussian's (12.5, three roundings) are rounded."""
+    worst = 0.0
+    for depth in 0.0101 + 13.7e-6 * np.arange(12):   # times all over a cell
+        w = phantoms.single_plane(depth=depth, lower=phantoms.BONE, n_el=4, n_s=1024, pitch=1e-3, fs=fs, n_cycles=n_cycles)
+        rf, quad, arr, launches = traced(ur, w, 40_000)
+        t = np.unique(arr["t"])
+        assert launches == 2 and t.size == 1 and np.bincount(arr["el"], minlength=4).min() >= 1024
+        s = n_cycles / (4 * w["array"]["f0"]) * fs
+        n = np.arange(1024)
+        n = n[np.abs(n - t[0]) <= 5 * s]
+        u = n - t[0]
+        env, phase = np.exp(-u * u / (2 * s * s)), 2 * np.pi * w["array"]["f0"] / fs * u
+        carrier = np.sin(phase) - 1j * np.cos(phase)
+        for e in range(4):
+            g = (rf[0, e] + 1j * quad[0, e])[n] / env
+            mid = np.abs(u) < s
+            amp = np.vdot(carrier[mid], g[mid]) / mid.sum()   # the row's amplitude
+            worst = max(worst, np.abs(g / amp - carrier).max())
+    h = 5 * s * 2 * w["array"]["f0"] / fs
+    assert worst <= (1.5 * np.pi * h + 3 * 12.5 + 8) * 2.0 ** -24
+
+
 def test_amplitudes_that_are_not_finite_keep_to_their_taps(ur):
     """A scatterer whose amplitude is NaN or infinite spoils the samples its pulses cover, no others."""
     w = workload(40e6, 1536, 5.0)
