@@ -998,14 +998,16 @@ void launch_binning(ur_ctx *c, float *d_rf, float *d_q, uint64_t n_arr) {
     B.rot32_c = (float)std::cos(kPi * 32.0 * (double)B.phase_per_sample);
     B.node_min = kNodeMin;
     B.node_chunk = kNodeChunk;
-    if (!c->nodes_ok) {   // the pulse's interpolation nodes, once per array
-        c->nodes = B;
-        ur::plan_bin_nodes(c->nodes, c->node_g, s_samples);
-        c->nodes_ok = true;
+    if (n_arr >= n_rows * kNodeMin) {
+        if (!c->nodes_ok) {   // the pulse's interpolation nodes, once per array
+            c->nodes = B;
+            ur::plan_bin_nodes(c->nodes, c->node_g, s_samples);
+            c->nodes_ok = true;
+        }
+        B.n_nodes = c->nodes.n_nodes;
+        std::copy(c->nodes.node, c->nodes.node + ur::kBinNodes, B.node);
+        std::copy(c->nodes.node_w, c->nodes.node_w + ur::kBinNodes, B.node_w);
     }
-    B.n_nodes = n_arr >= n_rows * kNodeMin ? c->nodes.n_nodes : 0;
-    std::copy(c->nodes.node, c->nodes.node + ur::kBinNodes, B.node);
-    std::copy(c->nodes.node_w, c->nodes.node_w + ur::kBinNodes, B.node_w);
     ck(cudaMemsetAsync(B.row_count, 0, sizeof(uint32_t) * n_rows, c->stream), "memset rows");
     ck(cudaMemsetAsync(B.row_fill, 0, sizeof(uint32_t) * n_rows, c->stream), "memset rows");
     c->phase_begin(UR_PHASE_SORT);

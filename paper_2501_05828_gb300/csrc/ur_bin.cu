@@ -385,6 +385,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_bin_nodes(const __grid_constan
 // the Gaussian and of the carrier), is 1e-6 RMS and 2.6e-6 to 6e-6 at most for pulses of 3 to 9 cycles at
 // 25 to 50 MHz; the bound takes 50 MHz x 5 cycles from 6 nodes (7.9e-6) to 7 (2.8e-7).
 constexpr double kNodeRel = 2.5e-6;
+constexpr double kNodeWeak = 3.7e-6;   // taps weaker than this (5 sigma) count as this strong
 
 constexpr int kNodeSmem = 226 << 10;   // most shared memory of a CTA
 
@@ -452,33 +453,51 @@ void plan_bin_nodes(BinP &B, BinNodeG &G, double s) {
     G.j_lo = (G.d_lo + kBinCell / 2 - (kBinCell - 1)) >> 2;
     G.n_j = ((G.d_hi + kBinCell / 2) >> 2) - G.j_lo + 1;
     if (G.n_j > kBinDist) return;
+    // The Gaussian at the taps -half .. half around x, outward from its peak by its ratios: two
+    // multiplications a tap (relative error below 1e-11).  A plan of fresh exponentials took 0.25 ms of
+    // a frame's host time.
+    constexpr int most = 4 * kBinDist;   // taps (half is below 2 kBinDist, see n_j above)
+    const int taps = 2 * half + 1;
+    const double step = std::exp(-1.0 / (s * s));
+    const auto gaussian = [&](double x, double *g) {
+        const double u = std::lround(x) - x, peak = std::exp(-u * u / (2.0 * s * s));
+        double *mid = g + half + std::lround(x);
+        double v = peak, ratio = std::exp(-(2.0 * u + 1.0) / (2.0 * s * s));
+        for (double *p = mid; p < g + taps; ++p, v *= ratio, ratio *= step) *p = v;
+        v = peak, ratio = std::exp((2.0 * u - 1.0) / (2.0 * s * s));
+        for (double *p = mid; p >= g; --p, v *= ratio, ratio *= step) *p = v;
+    };
+    constexpr int kOffsets = 17;   // arrival times over half a cell (the nodes are symmetric)
+    double at_t[kOffsets][most], at_x[kBinNodes][most];
+    for (int q = 0; q < kOffsets; ++q) gaussian(kBinCell / 2 * q / (kOffsets - 1.0), at_t[q]);
     for (int R = 5; R <= kBinNodes && !B.n_nodes; ++R) {
-        double x[kBinNodes], w[kBinNodes], worst = 0.0, worst_rel = 0.0;
+        double x[kBinNodes], w[kBinNodes];
         for (int k = 0; k < R; ++k) x[k] = kBinCell / 2 * std::cos((2 * k + 1) * 3.14159265358979323846 / (2 * R));
         for (int k = 0; k < R; ++k) {
             w[k] = 1.0;
             for (int m = 0; m < R; ++m)
                 if (m != k) w[k] /= x[k] - x[m];
+            gaussian(x[k], at_x[k]);
         }
-        // largest interpolation error of the unit-peak Gaussian over a cell and the pulse, and the largest
-        // relative to the tap itself where the nodes serve it
-        for (int q = 0; q <= 32; ++q) {
-            const double t = kBinCell * (q / 32.0 - 0.5);
-            double L[kBinNodes];
+        // the interpolation error of the unit-peak Gaussian over a cell and the pulse, and relative to the tap
+        // itself where the nodes serve it
+        bool good = true;
+        for (int q = 0; q < kOffsets && good; ++q) {
+            const double t = kBinCell / 2 * q / (kOffsets - 1.0);
+            double err[most];
+            for (int d = 0; d < taps; ++d) err[d] = -at_t[q][d];
             for (int k = 0; k < R; ++k) {
-                L[k] = w[k];
+                double L = w[k];
                 for (int m = 0; m < R; ++m)
-                    if (m != k) L[k] *= t - x[m];
+                    if (m != k) L *= t - x[m];
+                for (int d = 0; d < taps; ++d) err[d] += L * at_x[k][d];
             }
-            for (int d = -(int)B.K; d <= (int)B.K; ++d) {
-                const double g = std::exp(-(d - t) * (d - t) / (2.0 * s * s));
-                double v = -g;
-                for (int k = 0; k < R; ++k) v += L[k] * std::exp(-(d - x[k]) * (d - x[k]) / (2.0 * s * s));
-                worst = std::max(worst, std::fabs(v));
-                if (d >= G.d_lo && d <= G.d_hi) worst_rel = std::max(worst_rel, std::fabs(v) / g);
+            for (int d = 0; d < taps; ++d) {
+                const bool served = d >= G.d_lo + half && d <= G.d_hi + half;
+                good = good && std::fabs(err[d]) <= 2e-8 && (!served || std::fabs(err[d]) <= kNodeRel * std::max(at_t[q][d], kNodeWeak));
             }
         }
-        if (worst > 2e-8 || worst_rel > kNodeRel) continue;
+        if (!good) continue;
         B.n_nodes = R;
         for (int k = 0; k < R; ++k) {
             B.node[k] = (float)x[k];
