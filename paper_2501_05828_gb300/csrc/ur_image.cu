@@ -287,6 +287,8 @@ template <int KT>
 void launch_das_kt(const ImageP &I, const DasTile &D, dim3 grid, cudaStream_t s) {
     const size_t elems = (size_t)I.n_el * sizeof(ff) * (I.elem_xz ? 2 : 1);
     const size_t smem = elems > 256 * sizeof(float2) ? elems : 256 * sizeof(float2);
+    if (smem > 48 * 1024)   // convex arrays of more than 3072 elements; one value for every caller, up to 4096
+        cudaFuncSetAttribute(k_das<true, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * 2 * (int)sizeof(ff));
     if (I.elem_xz)
         k_das<true, KT><<<grid, 256, smem, s>>>(I, D);
     else
