@@ -1,7 +1,8 @@
 // Image formation: delay-and-sum of the analytic channel data with
 // coherent compounding over transmits, envelope, global maximum and log
-// compression.  Delays are evaluated in float-float so that the interpolation
-// position is exact to well below 1e-6 samples at any depth.
+// compression.  Transmit delays are evaluated in float-float, receive delays by a
+// square root corrected from its exact residual; both are held in 32.32 fixed point,
+// so that only the interpolation weight is rounded to FP32 (2^-25 samples).
 #include "ur_device.cuh"
 
 namespace ur {
@@ -15,17 +16,18 @@ __device__ __forceinline__ int ff_floor_i(ff a) {
 }
 
 // Delays in samples as 32.32 fixed point: a sum is two integer adds, the sample index is the
-// high word and the interpolation weight the low one.  hi + lo is a float-float (lo the tail, well
-// below one half): the fraction is rounded to 24 bits, as the weight it becomes, and stored in
-// units of 2^-30.  Valid for |hi| < kFixedMax.
+// high word and the interpolation weight the low one.  hi + lo is a float-float (lo the tail, below
+// one half): hi's distance to the nearest integer is exact, and it and the tail are rounded to 2^-31
+// each, so a delay is off by 2^-32 and only the weight by FP32's 2^-25 (with the fraction rounded to 24
+// bits as well, in units of 2^-30, the weight was off by up to 6e-8).  Valid for |hi| < kFixedMax.
 constexpr float kFixedMax = 2097152.f;   // 2^21 samples
 
 __device__ __forceinline__ long long to_fixed(float hi, float lo) {
     const float b = __fadd_rn(hi, 12582912.f);   // 1.5 x 2^23: the mantissa holds round(hi)
-    const float fr = __fadd_rn(__fsub_rn(hi, __fsub_rn(b, 12582912.f)), lo);   // the difference is exact
-    const int a = __float2int_rn(__fmul_rn(fr, 0x1p30f));
-    const int i = __float_as_int(b) - 0x4B400000 + (a >> 30);
-    return (long long)(((unsigned long long)(unsigned)i << 32) | ((unsigned)a << 2));
+    const float fr = __fsub_rn(hi, __fsub_rn(b, 12582912.f));   // exact
+    const int a = __float2int_rn(__fmul_rn(fr, 0x1p31f)) + __float2int_rn(__fmul_rn(lo, 0x1p31f));
+    const int i = __float_as_int(b) - 0x4B400000 + (a >> 31);
+    return (long long)(((unsigned long long)(unsigned)i << 32) | ((unsigned)a << 1));
 }
 
 __device__ __forceinline__ float rsqrt_approx(float a) {

@@ -19,6 +19,41 @@ def ur():
     return u
 
 
+@pytest.mark.parametrize("kind", ["plane", "diverging", "focused"])
+def test_weight_is_rounded_once(ur, kind):
+    """One element, samples 0 1 0 1 ...: where the delay's sample is even, the pixel's value is the
+    interpolation weight itself.  A weight in [0, 1) rounded once to FP32 is off by at most 2^-25;
+    the delays' own errors (32.32 fixed point, square roots) have to stay far below: 2^-28 in all."""
+    import torch
+    n_s = 8192
+    A = phantoms.array_params(1, n_s)
+    tx = {"plane": (ur.TX_PLANE, 0.2, 0.0), "diverging": (ur.TX_DIVERGING, 1e-3, -8e-3),
+          "focused": (ur.TX_FOCUSED, 2e-3, 0.3)}[kind]
+    x = np.linspace(-15e-3, 16e-3, 701).astype(np.float32)
+    z = np.linspace(2e-3, 0.14, 499).astype(np.float32)
+    rf = torch.zeros(1, 1, n_s, device="cuda")
+    rf[..., 1::2] = 1.0
+    sim = ur.Simulator(0)
+    sim.set_array(A)
+    sim.set_transmits([tx])
+    v = sim.beamform(rf, torch.zeros_like(rf), x, z)[0][..., 0].double().cpu().numpy()
+    q = A["fs"] / A["c_bf"]
+    X, Z = x.astype(np.float64)[None, :], z.astype(np.float64)[:, None]
+    R = np.sqrt(X * X + Z * Z)   # the element's centre is the origin
+    if kind == "plane":
+        a = float(np.float32(tx[1]))
+        T = X * np.sin(a) + Z * np.cos(a)
+    else:
+        vx, vz = float(np.float32(tx[1])), float(np.float32(tx[2]))
+        r, re = np.sqrt((X - vx) ** 2 + (Z - vz) ** 2), np.hypot(vx, vz)
+        T = r - re if kind == "diverging" else re + np.where(Z >= vz, r, -r)
+    tau = (T + R) * q
+    i0 = np.floor(tau)
+    even = (i0 % 2 == 0) & (tau > 0) & (tau < n_s - 1)
+    assert even.sum() > 100_000
+    assert np.abs(v - (tau - i0))[even].max() <= 2.0 ** -25 + 2.0 ** -28
+
+
 @pytest.mark.parametrize("n_el", [3072, 3073, 4096])
 def test_convex_arrays_of_many_elements(ur, n_el):
     """Every array that set_array takes can be beamformed.  Bar as in the tiles' tests."""
