@@ -98,6 +98,14 @@ __device__ __noinline__ float2 das_wide(const ImageP &I, int item, int k, int e0
 // SM), single transmits 51 and 55 against 52 us.
 constexpr long long kDasWarps = 10240;
 
+// Pixels along x of a warp: 16 in images of this width, else 8 (fewer in narrower images).  A warp of
+// 32 wastes up to half its lanes on the edge (33 columns of 64 elements x 8192 samples over 0.2 m, 7
+// transmits: slower than lanes along depth), and columns far apart share no cache lines along x.
+// Measured (us) at 32, 16, 8, 4: 31 transmits of 128 elements, 512 x 256 710, 705, 709, 730; 512 x 96
+// 326, 328, 389, 561; 383 x 301 645, 643, 643, 647; 128 x 1600 1179, 1068, 1025, 1019; 161 x 300 383, 358,
+// 338, 345; 97 x 700 621, 500, 459, 442; 33 x 2000 1065, 683, 524, 456; one transmit alike within 5 %.
+constexpr int kWideImage = 192;
+
 constexpr long long kNoTransmit = -(1ll << 62);   // with any receive delay: outside every recording
 
 // Samples a[0], b[0] if tau <= top, a[1], b[1] if tau's sample is not the last, else 0: predicated
@@ -122,7 +130,7 @@ __device__ __forceinline__ void gather(const float *a, const float *b, unsigned 
         : "l"(a), "l"(b), "l"(tau), "l"(top));
 }
 
-// How the image is cut up: a warp holds 1 << wx_log2 pixels along x (times 32 >> wx_log2 along z),
+// How the image is cut up: a warp holds 1 << wx_log2 pixels along x and 32 >> wx_log2 along z,
 // and `split` warps of a CTA share a group of pixels, each summing its part of the elements.
 struct DasTile {
     int wx_log2, split, tiles_x;
@@ -132,8 +140,8 @@ struct DasTile {
 //
 // Bound by issue slots and, next, by the L1 reads of the four gathers per (pixel, element,
 // transmit) term.  Lanes run along x: neighbouring pixels of a row read samples at most a lateral
-// step apart (0.5 on average on the 512 x 256 image of 128 elements), so a gather touches one or
-// two cache lines, where lanes along depth are 2 dz fs / c = 12 samples apart and touch one sector
+// step apart (0.5 on average on the 512 x 256 image of 128 elements), so a row's gather touches one
+// or two cache lines, where lanes along depth are 2 dz fs / c = 12 samples apart and touch one sector
 // each.  A CTA's warps take consecutive rows of one x range, which share lines the same way.  The
 // receive delay is formed once per (pixel, element) and serves KT transmits; times are 32.32 fixed
 // point, so a term adds, splits and compares integers.  512 x 256 image of 128 elements x 3200 samples,
@@ -303,7 +311,7 @@ void launch_das(const ImageP &I, cudaStream_t s) {
     const int images = I.img_items ? I.n_images : 1;
     DasTile D;
     D.wx_log2 = 0;   // narrow images: as many pixels along x as there are, the warp's other lanes along z
-    while (D.wx_log2 < 5 && (1 << D.wx_log2) < I.nx) ++D.wx_log2;
+    while (D.wx_log2 < (I.nx >= kWideImage ? 4 : 3) && (1 << D.wx_log2) < I.nx) ++D.wx_log2;
     D.tiles_x = (I.nx + (1 << D.wx_log2) - 1) >> D.wx_log2;
     // small images: warps share a pixel's elements until there are about kDasWarps of them
     const long long warps = (((long long)I.nx * I.nz + 31) >> 5) * images;

@@ -54,6 +54,33 @@ def test_weight_is_rounded_once(ur, kind):
     assert np.abs(v - (tau - i0))[even].max() <= 2.0 ** -25 + 2.0 ** -28
 
 
+def test_columns_far_apart_and_past_a_warp(ur):
+    """33 columns over 0.2 m cost no more each than 12 do: neither the lanes of a second warp without
+    pixels nor gathers without a shared cache line (1.4 times as much with warps of 32 columns)."""
+    import torch
+    A = phantoms.array_params(64, 8192)
+    sim = ur.Simulator(0)
+    sim.set_array(A)
+    sim.set_plane_waves(np.deg2rad(np.linspace(-10, 10, 31)).astype(np.float32))
+    rf, quad = (torch.randn(31, 64, 8192, device="cuda") for _ in range(2))
+    z = torch.linspace(1e-3, 0.15, 2000, device="cuda")
+
+    def time(nx):
+        x = torch.linspace(-0.1, 0.1, nx, device="cuda")
+        out = [torch.empty(2000, nx, 2, device="cuda")] + [torch.empty(2000, nx, device="cuda") for _ in range(2)]
+        t = []
+        for _ in range(9):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            sim.beamform(rf, quad, x, z, 60.0, *out)
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    assert time(33) / 33 <= 1.15 * time(12) / 12
+
+
 @pytest.mark.parametrize("n_el", [3072, 3073, 4096])
 def test_convex_arrays_of_many_elements(ur, n_el):
     """Every array that set_array takes can be beamformed.  Bar as in the tiles' tests."""
