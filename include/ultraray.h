@@ -384,9 +384,10 @@ ur_status ur_graph_launch(ur_ctx *ctx);
  * 2 r_s when every boundary is a smooth plane z = c or cylinder along y (plane waves of a
  * linear array then never gain a y component, so thin y cells cost no visits and hold fewer
  * scatterers); 4, 2, 2 r_s when such boundaries are rough; 14, 14, 2 r_s with spheres or
- * triangles; wider where scatterers are sparser, narrower where they are denser.  block (multiple of 32, <= 256), blocks_per_sm and
- * resolve_batch (1..32: the tracer starts new rays once this many lanes of a warp
- * are without one; default 18, 10 in the extended tracers) apply at the next trace. */
+ * triangles; wider where scatterers are sparser, narrower where they are denser (by the density of
+ * their bounding box or, where they cluster in it, the clusters').  block (multiple of 32, <= 256),
+ * blocks_per_sm and resolve_batch (1..32: the tracer starts new rays once this many lanes of a
+ * warp are without one; default 18, 10 in the extended tracers) apply at the next trace. */
 typedef struct {
     float cell_xy, cell_z;
     int32_t block, blocks_per_sm, resolve_batch;

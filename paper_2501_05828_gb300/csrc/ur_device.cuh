@@ -580,7 +580,16 @@ struct GridBuildP {
     float4 *refs;
     float *amp;
 };
-void launch_bbox(const float4 *scat, int n, float *lohi /* 6 floats as ordered ints */, cudaStream_t s);
+constexpr uint32_t kCoarseMax = 1u << 18;   // most coarse cells
+struct CoarseGrid {
+    unsigned int lohi[6];       // the scatterers' box as ordered ints (min x, y, z, max x, y, z)
+    unsigned long long pairs;   // ordered pairs that share a coarse cell
+    uint32_t cells, pad;
+    uint32_t count[kCoarseMax];
+};
+void launch_bbox(const float4 *scat, int n, unsigned int *lohi, cudaStream_t s);
+// Pairs and cells of every stride-th scatterer in the box (pairs and count zeroed before); 2 kernels.
+void launch_coarse(const float4 *scat, int n, int stride, float r_s, float cell, CoarseGrid *C, cudaStream_t s);
 void launch_grid_count(const GridBuildP &G, cudaStream_t s);
 void launch_scan_u32(const uint32_t *in, uint32_t *out, uint32_t *block_sums, uint32_t n, cudaStream_t s);
 void launch_grid_fill(const GridBuildP &G, cudaStream_t s);

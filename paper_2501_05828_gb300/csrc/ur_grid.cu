@@ -35,6 +35,54 @@ __global__ void k_bbox(const float4 *scat, int n, unsigned int *lohi) {
     }
 }
 
+__device__ __forceinline__ float unordered(unsigned int u) {
+    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+
+// Scatterers (every stride-th) per cell of a coarse grid over their box (as k_bbox left it: the host need
+// not read it first): cells of `cell` capture radii, wider where there would be more than kCoarseMax.
+__global__ void k_coarse_count(const float4 *scat, int n, int stride, float r_s, float cell, CoarseGrid *C) {
+    __shared__ float s_lo[3], s_inv_h[3];
+    __shared__ int s_dim[3];
+    if (threadIdx.x == 0) {
+        float side[3], dim[3];
+        for (int a = 0; a < 3; ++a) {
+            s_lo[a] = unordered(C->lohi[a]);
+            side[a] = fmaxf(2.f, (unordered(C->lohi[3 + a]) - s_lo[a]) / r_s);
+            if (!(side[a] < 1e9f)) side[a] = 1e9f;   // coordinates that are not finite: refused by the host
+        }
+        for (float h = cell;; h *= 1.5f) {
+            for (int a = 0; a < 3; ++a) dim[a] = fmaxf(1.f, ceilf(side[a] / h));
+            if (dim[0] * dim[1] * dim[2] <= (float)kCoarseMax) break;
+        }
+        for (int a = 0; a < 3; ++a) {
+            s_dim[a] = (int)dim[a];
+            s_inv_h[a] = dim[a] / (side[a] * r_s);
+        }
+        if (blockIdx.x == 0) C->cells = (uint32_t)(s_dim[0] * s_dim[1] * s_dim[2]);
+    }
+    __syncthreads();
+    const int taken = (n - 1) / stride + 1;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < taken; k += gridDim.x * blockDim.x) {
+        const float4 p = scat[(size_t)k * stride];
+        const int x = min(max((int)((p.x - s_lo[0]) * s_inv_h[0]), 0), s_dim[0] - 1);
+        const int y = min(max((int)((p.y - s_lo[1]) * s_inv_h[1]), 0), s_dim[1] - 1);
+        const int z = min(max((int)((p.z - s_lo[2]) * s_inv_h[2]), 0), s_dim[2] - 1);
+        atomicAdd(&C->count[(x * s_dim[1] + y) * s_dim[2] + z], 1u);
+    }
+}
+
+// The ordered pairs of those scatterers that share a cell.
+__global__ void k_coarse_pairs(CoarseGrid *C) {
+    unsigned long long s = 0;
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C->cells; c += gridDim.x * blockDim.x) {
+        const unsigned long long k = C->count[c];
+        if (k > 1) s += k * (k - 1);
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd(&C->pairs, s);
+}
+
 // Columns (x, y) whose cells a scatterer at p is referenced from, and its z cell.
 __device__ __forceinline__ void cell_range(const GridBuildP &G, float4 p, int3 &c0, int3 &c1) {
     c0.x = min(max((int)floorf((p.x - G.r_m - G.lo.x) * G.inv_h.x), 0), G.dim.x - 1);
@@ -148,8 +196,13 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_apply(const uint32_t *in, u
 
 }  // namespace
 
-void launch_bbox(const float4 *scat, int n, float *lohi, cudaStream_t s) {
-    k_bbox<<<min(1024, (n + 255) / 256 + 1), 256, 0, s>>>(scat, n, reinterpret_cast<unsigned int *>(lohi));
+void launch_bbox(const float4 *scat, int n, unsigned int *lohi, cudaStream_t s) {
+    k_bbox<<<min(1024, (n + 255) / 256 + 1), 256, 0, s>>>(scat, n, lohi);
+}
+
+void launch_coarse(const float4 *scat, int n, int stride, float r_s, float cell, CoarseGrid *C, cudaStream_t s) {
+    k_coarse_count<<<min(1024, n / stride / 256 + 1), 256, 0, s>>>(scat, n, stride, r_s, cell, C);
+    k_coarse_pairs<<<128, 256, 0, s>>>(C);
 }
 
 void launch_grid_count(const GridBuildP &G, cudaStream_t s) {
