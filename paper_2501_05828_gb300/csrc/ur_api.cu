@@ -107,7 +107,6 @@ constexpr int kCoarseScat = 1 << 16;  // of this many scatterers at most, evenly
 // scene.  83 % of the layered frame's reference tests came from such segments.
 constexpr float kCellFine[3] = {0.5f, 0.5f, 10.f};
 constexpr double kFineMaxCells = (double)(1u << 24);
-constexpr int kResolveBatch = 10;   // where the autotuner starts (ur_tuning::resolve_batch)
 
 struct SceneData {
     bool ok = false;
@@ -963,6 +962,15 @@ void size_trace_buffers(ur_ctx *c, uint64_t cap, bool dbg) {
     c->grow(c->n_work, 2 * sizeof(uint32_t));
 }
 
+// Other transmit kinds than plane waves, and mixing, run the extended tracer.
+void transmit_needs(const ur_ctx *c, const ur::TraceP &P, bool &point_waves, bool &emit) {
+    point_waves = emit = P.mix_tx > 0;
+    for (const ur::ItemP &it : c->items) {
+        point_waves = point_waves || it.kind != UR_TX_PLANE;
+        emit = emit || it.kind == UR_TX_SYNTHETIC;
+    }
+}
+
 void launch_trace_kernel(ur_ctx *c, ur::TraceP &P, bool dbg, uint2 *arr_dbg) {
     c->rec_key.valid = false;   // the arrival buffers are about to change
     P.arr = (uint4 *)c->arrivals.p;
@@ -971,11 +979,8 @@ void launch_trace_kernel(ur_ctx *c, ur::TraceP &P, bool dbg, uint2 *arr_dbg) {
     ck(cudaMemsetAsync(P.arr_count, 0, 8 * sizeof(unsigned long long), c->stream), "memset counters");
     c->phase_begin(UR_PHASE_TRACE);
     if (P.mix_list) ck(ur::launch_mix_plan(c->mix, c->sms, c->stream), "mixed ray order");
-    bool point_waves = P.mix_tx > 0, emit = P.mix_tx > 0;   // other transmit kinds and mixing: extended tracer
-    for (const ur::ItemP &it : c->items) {
-        point_waves = point_waves || it.kind != UR_TX_PLANE;
-        emit = emit || it.kind == UR_TX_SYNTHETIC;
-    }
+    bool point_waves, emit;
+    transmit_needs(c, P, point_waves, emit);
     bool split = false;
     for (int q = 0; q < P.n_scenes; ++q) split = split || P.S[q].split_sampling != 0;
     if (split && (point_waves || P.radius > 0.f))
@@ -1877,14 +1882,19 @@ ur_status ur_autotune(ur_ctx *c, int scene, uint64_t n_rays, uint64_t seed, int 
         if (cur.cell_xy <= 0.f) cur.cell_xy = default_cell(sd, 0);
         if (cur.cell_y <= 0.f) cur.cell_y = default_cell(sd, 1);
         if (cur.cell_z <= 0.f) cur.cell_z = default_cell(sd, 2);
-        if (cur.resolve_batch <= 0) cur.resolve_batch = kResolveBatch;
+        if (cur.resolve_batch <= 0) {
+            const ur::TraceP P = make_trace_params(c, seed, max_b, max_path);
+            bool point_waves, emit;
+            transmit_needs(c, P, point_waves, emit);
+            cur.resolve_batch = ur::trace_idle_min(P, point_waves, emit);
+        }
         if (cur.blocks_per_sm <= 0) cur.blocks_per_sm = ur::trace_occupancy(256, false);
         float t_cur = measure(cur);
-        // coordinate descent over the knobs
+        // coordinate descent over the knobs, from what an untuned trace runs with
         const float z_mult[] = {2.f, 4.f, 8.f};
         const float xy_mult[] = {2.f, 4.f, 6.f, 9.f, 14.f, 20.f, 30.f};
-        const float y_mult[] = {0.2f, 0.3f, 0.5f, 1.f, 2.f, 4.f, 9.f, 14.f, 20.f};
-        const int batches[] = {1, 6, 10, 14, 20};
+        const float y_mult[] = {0.15f, 0.2f, 0.3f, 0.5f, 1.f, 2.f, 4.f, 9.f, 14.f, 20.f};
+        const int batches[] = {1, 6, 10, 14, 18, 22};
         for (int pass = 0; pass < 2; ++pass) {
             for (float m : z_mult) {
                 ur_tuning t = cur;

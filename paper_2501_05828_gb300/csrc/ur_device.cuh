@@ -509,6 +509,7 @@ __device__ __forceinline__ float cross2(float3 v, float3 n) {
 void launch_trace(const TraceP &P, bool debug, int block, int grid, cudaStream_t s, bool point_waves,
                   bool emit);
 int trace_occupancy(int block, bool debug);   // resident tracer CTAs per SM
+int trace_idle_min(const TraceP &P, bool point_waves, bool emit);   // that launch's default for resolve_batch
 
 // Path-replay adjoint: loss sensitivities in, parameter gradients out.
 struct AdjP {

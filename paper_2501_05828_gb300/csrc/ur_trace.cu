@@ -12,15 +12,32 @@ int trace_occupancy(int block, bool debug) {
     return n > 0 ? n : 1;
 }
 
+namespace {
+
+// What a launch's scenes, array and transmits ask of the tracer.
+struct Needs {
+    bool split = false, mesh = false, rough;
+    Needs(const TraceP &P, bool point_waves) : rough(point_waves || P.radius > 0.f) {   // convex arrays: extended tracer
+        for (int q = 0; q < P.n_scenes && q < kMaxScenes; ++q) {
+            split = split || P.S[q].split_sampling != 0;
+            mesh = mesh || P.S[q].n_tri > 0;
+            for (int b = 0; b < P.S[q].n_bnd; ++b) rough = rough || P.S[q].bnd[b].alpha > 0.f;
+        }
+    }
+    bool extended(bool emit) const { return rough || mesh || emit; }
+};
+
+}  // namespace
+
+int trace_idle_min(const TraceP &P, bool point_waves, bool emit) {
+    return Needs(P, point_waves).extended(emit) ? kIdleMinExtended : kIdleMin;
+}
+
 template <int ONE>
 void launch_trace_of(const TraceP &P, bool debug, int block, int grid, cudaStream_t s, bool point_waves, bool emit) {
-    bool split = false, mesh = false, rough = point_waves || P.radius > 0.f;   // convex arrays: extended tracer
-    for (int q = 0; q < P.n_scenes && q < kMaxScenes; ++q) {
-        split = split || P.S[q].split_sampling != 0;
-        mesh = mesh || P.S[q].n_tri > 0;
-        for (int b = 0; b < P.S[q].n_bnd; ++b) rough = rough || P.S[q].bnd[b].alpha > 0.f;
-    }
-    if (rough || mesh || emit) {
+    const Needs needs(P, point_waves);
+    const bool split = needs.split, mesh = needs.mesh;
+    if (needs.extended(emit)) {
         const int cvx = P.radius > 0.f ? kGeoConvex : 0;
         if (mesh) {
             if (cvx) launch_extended<kGeoConvex | kGeoMesh | kGeoEmit | ONE>(P, debug, block, grid, s);
