@@ -226,7 +226,8 @@ ur_status ur_set_transmit_mixing(ur_ctx *ctx, int enabled);
  * rf + j quad, both [n_tx][n_el][n_s] float32 (overwritten).  Ray i of
  * transmit k leaves element i mod n_el at a uniformly random point of its
  * face; all randomness is Philox4x32-10 keyed by (seed, i, k, event), so the
- * result is a pure function of the arguments.  max_bounces <= 127 boundary
+ * arrivals are a pure function of the arguments; the channel data are so up to the
+ * order of their FP32 sums, which differs from run to run.  max_bounces <= 127 boundary
  * interactions per path, max_path_m total path length.  st may be NULL.
  * Errors: UR_ERR_STATE, UR_ERR_INVALID_ARG, UR_ERR_OOM, UR_ERR_CUDA. */
 ur_status ur_trace(ur_ctx *ctx, uint64_t n_rays_per_tx, uint64_t seed, int max_bounces,
@@ -357,7 +358,11 @@ ur_status ur_batch_plan(ur_ctx *ctx, const ur_batch_item *items, int n_items, ui
 
 /* Trace and deposit the planned batch into rf, quad [n_items][n_el][n_s]
  * (device memory).  Asynchronous, allocates nothing and may be captured into
- * a graph (ur_graph_begin).  If the queue overflows, ur_batch_status reports it. */
+ * a graph (ur_graph_begin).  If the queue overflows, ur_batch_status reports it.
+ * Rows of 1024 arrivals or more are deposited through interpolation nodes (the same
+ * samples to FP32 rounding) where the call holds that many per row on average: ur_trace
+ * counts its arrivals, a batch goes by its queue's size, which earlier and larger traces
+ * of the context may have grown. */
 ur_status ur_batch_trace(ur_ctx *ctx, uint64_t seed, int max_bounces, float max_path_m, float *rf, float *quad);
 
 /* Synchronise and report the last trace: arrivals produced and counters.
@@ -366,7 +371,9 @@ ur_status ur_batch_status(ur_ctx *ctx, uint64_t *n_arrivals, ur_stats *st);
 
 /* Delay-and-sum of the planned batch: image i compounds all items of the i-th
  * scene present (outputs [n_images][nz][nx], device memory, each nullable).
- * Asynchronous and capturable. */
+ * Asynchronous and capturable.  The order of a pixel's sums follows from the image's size,
+ * the number of images and their transmits, so an image's last bits may differ from those of
+ * ur_beamform or of another batch (repeated calls give the same bits). */
 ur_status ur_batch_beamform(ur_ctx *ctx, const float *rf, const float *quad, float dyn_range_db,
                             float *iq, float *env, float *db);
 
