@@ -64,19 +64,36 @@ FP32_LANES_PER_SM = 128
 # DRAM traffic of the tracer kernel (dram__bytes_read.sum + dram__bytes_write.sum) and its warp
 # instructions (smsp__inst_executed.sum), from one single-pass ncu capture of the benchmarked
 # 1e7-ray launch, per primary ray; valid only while the tracer sources hash to `src_sha`.
-TRACE_TRAFFIC = {"src_sha": "079027dccbf37cf5", "bytes_per_ray": 6.555, "warp_inst_per_ray": 262.0}
+TRACE_TRAFFIC = {"src_sha": "37bf3dcea057bda4", "bytes_per_ray": 6.558, "warp_inst_per_ray": 262.2}
 
 
 def tracer_sha():
-    """Hash of the tracer kernel's sources and of the default grid cells (which set its traffic)."""
+    """Hash of the tracer kernel's sources and of what chooses the default grid cells (which set its
+    traffic): the cell rules' constants, the rule and the grid's construction."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2501_05828_gb300", "csrc")
-    for f in ("ur_trace.cuh", "ur_trace.cu", "ur_device.cuh"):
+    for f in ("ur_trace.cuh", "ur_trace.cu", "ur_device.cuh", "ur_grid.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "ur_api.cu"), "rb") as fh:
-        h.update(b"".join(l for l in fh if l.startswith(b"constexpr float kCell")))
+        api = fh.read()
+    h.update(b"\n".join(l for l in api.split(b"\n") if l.startswith(b"constexpr ") and (b" kCell" in l or b" kCoarse" in l)))
+    for name in (b"struct CellRule {", b"float default_cell(const SceneData &sd, int a) {",
+                 b"void build_grid(ur_ctx *c, SceneData &sd, const float *src) {"):
+        begin = api.index(b"\n" + name)
+        h.update(api[begin:api.index(b"\n}", begin)])
     return h.hexdigest()[:16]
+
+
+# Warp instructions (smsp__inst_executed.sum) of the node deposit of the benchmarked frame, per arrival,
+# from the same kind of capture; valid only while its source hashes to `src_sha`.
+NODE_DEPOSIT = {"src_sha": "3e16fe30f16e2d89", "warp_inst_per_arrival": 62.8}
+
+
+def deposit_sha():
+    """Hash of the deposit kernels' source."""
+    with open(os.path.join(ROOT, "paper_2501_05828_gb300", "csrc", "ur_bin.cu"), "rb") as fh:
+        return hashlib.sha256(fh.read()).hexdigest()[:16]
 
 
 def taps_per_arrival(arr):
@@ -103,19 +120,25 @@ def issue_slots(rays, t_launch, n_sm, sm_mhz):
             "peak_note": "%d SMs x 4 schedulers x 1 warp instruction per clock x %.0f MHz" % (n_sm, sm_mhz)}
 
 
-def binning_roofline(st, arr, phase_ms, alu_peak, peaks, n_sm, sm_mhz):
-    """Binning of one frame: the deposit kernels against the FP32 ALU peak (FLOPS_PER_TAP per pulse
-    tap of the method, whether a row is deposited tap by tap or through interpolation nodes), and
-    the counting sort's algorithmic bytes (arrival read by count and scatter, sorted write) against
-    HBM."""
+def binning_roofline(st, arr, phase_ms, alu_peak, peaks, n_sm, sm_mhz, benchmarked):
+    """Binning of one frame: the deposit against the issue slots that bound it (warp instructions
+    captured per arrival with ncu on the benchmarked frame, whose rows all go through interpolation
+    nodes; None for other frames or sources), the method's own arithmetic (FLOPS_PER_TAP per pulse
+    tap, which nodes do not evaluate one by one) for reference, and the counting sort's algorithmic
+    bytes (arrival read by count and scatter, sorted write) against HBM."""
     taps = st["arrivals"] * taps_per_arrival(arr)
     t_dep = phase_ms.get("deposit", float("nan")) * 1e-3
     t_sort = phase_ms.get("sort", float("nan")) * 1e-3
-    ach = taps * FLOPS_PER_TAP / t_dep / 1e12
+    got = None
+    if benchmarked and NODE_DEPOSIT["src_sha"] == deposit_sha():
+        got = NODE_DEPOSIT["warp_inst_per_arrival"] * st["arrivals"] / t_dep
+    peak = n_sm * 4 * sm_mhz * 1e6
     sort_bytes = st["arrivals"] * 48
     hbm = peaks.get("hbm_gbs", 6800.0)
-    return {"bound": "alu", "kernel": "k_bin_deposit + k_bin_nodes", "achieved": ach, "peak": alu_peak, "unit": "TFLOP/s",
-            "frac": ach / alu_peak, "traffic": None, "algorithmic_flops_per_launch": taps * FLOPS_PER_TAP,
+    return {"bound": "issue", "kernel": "k_bin_deposit + k_bin_nodes", "achieved": got, "peak": peak,
+            "unit": "warp instructions/s", "frac": got / peak if got is not None else None, "traffic": None,
+            "method_flops_per_launch": taps * FLOPS_PER_TAP,
+            "method_tflops": taps * FLOPS_PER_TAP / t_dep / 1e12, "alu_peak_tflops": alu_peak,
             "deposit_ms_per_launch": t_dep * 1e3,
             "sort": {"bound": "hbm", "kernels": "k_bin_count + k_bin_plan + k_bin_scatter",
                      "algorithmic_bytes": sort_bytes, "achieved": sort_bytes / t_sort / 1e9, "peak": hbm,
@@ -399,7 +422,8 @@ def run_ours(args, rank, world, local_rank):
                          "algorithmic_flops_per_launch": trace_flops(st),
                          "issue_slots": issue_slots(N * n_tx, t_launch, props.multi_processor_count, sm_mhz)
                          if traffic is not None else None},
-            "roofline_binning": binning_roofline(st, A, phase_ms, peak, peaks, props.multi_processor_count, sm_mhz),
+            "roofline_binning": binning_roofline(st, A, phase_ms, peak, peaks, props.multi_processor_count, sm_mhz,
+                                                 args.workload == "layered"),
             "stats_per_frame": st,
             "gpu_launches": launches,
             "e2e": {"value": whole_job_rate(N * n_tx, world, e2e_s), "unit": UNIT, "h2d_bytes_per_step": int(h2d),
