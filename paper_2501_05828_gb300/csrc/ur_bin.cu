@@ -250,11 +250,13 @@ __global__ void __launch_bounds__(512) k_bin_deposit(const BinP B) {
 // tap (14 instead of 202).  Each sample then sums g over the nodes of the cells around it once.  Only
 // taps inside the pulse's cut |n - t| <= K for every t of a cell go through the nodes; the up to 5 others
 // of an arrival are deposited one by one, so the cut stays where it is.
-// The Gaussian's values come from the kernel's constants.  Bound by the chains of shared-memory
-// atomics on the same cells (echoes of a plane or a scatterer share their time).  Layered frame
-// (2.27M arrivals, 128 rows) 412 -> 240 us, 4096 rows of 1.8k arrivals 1239 -> 690 us; error of the layered
-// frame's channel data against 64 bits 1.4e-6 -> 3.0e-7.  Tap by tap stays the better one below about
-// 1000 arrivals per row (680 per row: 63 us against 89).
+// The Gaussian's values come from the kernel's constants.  Bound by issue on the layered frame (82 % of
+// the slots, 63 warp instructions per arrival; shared-memory latency next), and by the chains of
+// shared-memory atomics where arrivals of other times crowd into the same cells: there tap by tap
+// is faster, but the host does not know (one focused transmit of 2e6 rays 70 us tap by tap, 200 this
+// way).  Layered frame (2.27M arrivals, 128 rows) 412 -> 240 us, 4096 rows of 1.8k arrivals 1239 -> 690 us;
+// error of the layered frame's channel data against 64 bits 1.4e-6 -> 3.0e-7.  Tap by tap stays the
+// better one below about 1000 arrivals per row (680 per row: 63 us against 89).
 constexpr int kNodeThreads = 512;
 
 // Samples before (and after) the row that its cells cover, a multiple of the cell; cells of a row.
