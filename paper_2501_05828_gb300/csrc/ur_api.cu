@@ -86,8 +86,8 @@ constexpr uint32_t kNodeChunk = 4096;
 // at least the scatterers' own (that of their coarse cells) over `contrast`; the measured phantoms' is 1
 // (layered) and 3 (bone inside its box) times the box's.  50k scatterers in 8 x 5 x 8 mm and one 0.3 m away,
 // 2e6 rays at 10 degrees, by the box alone, with this, and with the best uniform cells (us): among planes
-// 6482, 2370, 1656; the same with rough bone 8679, 2039, 2057; in the bone scene 57191, 2509, 2575.
-// (Counting the coarse cells takes 10 to 15 us of an upload.)
+// 6482, 2228, 1656; the same with rough bone 8679, 2438, 2057; in the bone scene 57191, 2525, 2575.
+// (Counting the coarse cells takes 10 to 20 us of an upload.)
 struct CellRule {
     float cell[3];
     float density;    // scatterers per r_s^3 the sizes were measured at
@@ -98,8 +98,8 @@ struct CellRule {
 constexpr CellRule kCellSlab = {{9.f, 0.15f, 2.f}, 4.4e-3f, 0.5f, 0.4f, 8.f, 20.f};
 constexpr CellRule kCellRough = {{4.f, 2.f, 2.f}, 4.4e-3f, 1.f / 3.f, 0.5f, 6.f, 20.f};
 constexpr CellRule kCellIso = {{14.f, 14.f, 2.f}, 1.1e-3f, 1.f / 3.f, 0.25f, 6.f, 5.f};
-constexpr float kCoarseCell = 16.f;   // coarse cells in r_s,
-constexpr int kCoarseScat = 1 << 16;  // of this many scatterers at most, evenly taken
+constexpr float kCoarseCell = 16.f;    // coarse cells in r_s,
+constexpr int kCoarseScat = 1 << 15;   // of this many scatterers at most, evenly taken
 // Fine columns (x, y, z in r_s) for exactly vertical segments (every 0-degree plane-wave ray until
 // it meets a tilted boundary, and every normal-incidence echo): such a segment stays in one
 // column, so narrow columns cost it no steps and hold (0.5 + 2)^2 / pi = 2x the scatterers of
@@ -445,7 +445,10 @@ void build_grid(ur_ctx *c, SceneData &sd, const float *src) {
     for (int a = 0; a < 3; ++a) box *= std::max(2.0, ((double)hi[a] - (double)lo[a]) / (double)sd.r_s);
     const ur::CoarseGrid *hc = (const ur::CoarseGrid *)hb;   // its head
     sd.density = (float)((double)n / box);
-    sd.own_density = (float)((double)hc->pairs / taken * stride * hc->cells / box);
+    const double cells = (double)hc->dim[0] * hc->dim[1] * hc->dim[2];
+    double pairs = (double)hc->pairs;   // of hashed cells without those that only share a counter
+    if (cells > (double)ur::kCoarseMax) pairs = std::max(0.0, pairs - (double)taken * (taken - 1.0) / ur::kCoarseMax);
+    sd.own_density = (float)(pairs / taken * stride * cells / box);
     float h_x = c->tune.cell_xy > 0.f ? c->tune.cell_xy : default_cell(sd, 0);
     float h_y = c->tune.cell_y > 0.f ? c->tune.cell_y : default_cell(sd, 1);
     float h_z = c->tune.cell_z > 0.f ? c->tune.cell_z : default_cell(sd, 2);

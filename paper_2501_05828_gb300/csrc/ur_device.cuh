@@ -583,11 +583,11 @@ struct GridBuildP {
     float4 *refs;
     float *amp;
 };
-constexpr uint32_t kCoarseMax = 1u << 18;   // most coarse cells
+constexpr uint32_t kCoarseMax = 1u << 16;   // most coarse cells with a counter of their own
 struct CoarseGrid {
     unsigned int lohi[6];       // the scatterers' box as ordered ints (min x, y, z, max x, y, z)
-    unsigned long long pairs;   // ordered pairs that share a coarse cell
-    uint32_t cells, pad;
+    unsigned long long pairs;   // ordered pairs that share a counter
+    int dim[3], pad;            // coarse cells along each axis; more than kCoarseMax share counters by a hash
     uint32_t count[kCoarseMax];
 };
 void launch_bbox(const float4 *scat, int n, unsigned int *lohi, cudaStream_t s);

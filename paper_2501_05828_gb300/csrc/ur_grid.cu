@@ -40,42 +40,42 @@ __device__ __forceinline__ float unordered(unsigned int u) {
 }
 
 // Scatterers (every stride-th) per cell of a coarse grid over their box (as k_bbox left it: the host need
-// not read it first): cells of `cell` capture radii, wider where there would be more than kCoarseMax.
+// not read it first): cells of about `cell` capture radii.  Where there are more than kCoarseMax of them
+// (a few scatterers far away stretch the box), cells are hashed to the counters; few are occupied.
 __global__ void k_coarse_count(const float4 *scat, int n, int stride, float r_s, float cell, CoarseGrid *C) {
     __shared__ float s_lo[3], s_inv_h[3];
     __shared__ int s_dim[3];
     if (threadIdx.x == 0) {
-        float side[3], dim[3];
         for (int a = 0; a < 3; ++a) {
             s_lo[a] = unordered(C->lohi[a]);
-            side[a] = fmaxf(2.f, (unordered(C->lohi[3 + a]) - s_lo[a]) / r_s);
-            if (!(side[a] < 1e9f)) side[a] = 1e9f;   // coordinates that are not finite: refused by the host
+            float side = fmaxf(2.f, (unordered(C->lohi[3 + a]) - s_lo[a]) / r_s);
+            if (!(side < 1e9f)) side = 1e9f;   // or coordinates that are not finite: refused by the host
+            s_dim[a] = max(1, (int)ceilf(side / cell));
+            s_inv_h[a] = (float)s_dim[a] / (side * r_s);
+            if (blockIdx.x == 0) C->dim[a] = s_dim[a];
         }
-        for (float h = cell;; h *= 1.5f) {
-            for (int a = 0; a < 3; ++a) dim[a] = fmaxf(1.f, ceilf(side[a] / h));
-            if (dim[0] * dim[1] * dim[2] <= (float)kCoarseMax) break;
-        }
-        for (int a = 0; a < 3; ++a) {
-            s_dim[a] = (int)dim[a];
-            s_inv_h[a] = dim[a] / (side[a] * r_s);
-        }
-        if (blockIdx.x == 0) C->cells = (uint32_t)(s_dim[0] * s_dim[1] * s_dim[2]);
     }
     __syncthreads();
+    const bool own = (double)s_dim[0] * s_dim[1] * s_dim[2] <= (double)kCoarseMax;
     const int taken = (n - 1) / stride + 1;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < taken; k += gridDim.x * blockDim.x) {
         const float4 p = scat[(size_t)k * stride];
         const int x = min(max((int)((p.x - s_lo[0]) * s_inv_h[0]), 0), s_dim[0] - 1);
         const int y = min(max((int)((p.y - s_lo[1]) * s_inv_h[1]), 0), s_dim[1] - 1);
         const int z = min(max((int)((p.z - s_lo[2]) * s_inv_h[2]), 0), s_dim[2] - 1);
-        atomicAdd(&C->count[(x * s_dim[1] + y) * s_dim[2] + z], 1u);
+        uint32_t c = ((uint32_t)x * s_dim[1] + y) * s_dim[2] + z;
+        if (!own) {   // odd multipliers, the high bits folded down
+            c = (uint32_t)x * 0x9E3779B1u + (uint32_t)y * 0x85EBCA77u + (uint32_t)z * 0xC2B2AE3Du;
+            c = (c ^ c >> 15) * 0x2C1B3C6Du >> 16;
+        }
+        atomicAdd(&C->count[c], 1u);
     }
 }
 
-// The ordered pairs of those scatterers that share a cell.
+// The ordered pairs of those scatterers that share a counter.
 __global__ void k_coarse_pairs(CoarseGrid *C) {
     unsigned long long s = 0;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C->cells; c += gridDim.x * blockDim.x) {
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < kCoarseMax; c += gridDim.x * blockDim.x) {
         const unsigned long long k = C->count[c];
         if (k > 1) s += k * (k - 1);
     }
