@@ -64,7 +64,7 @@ FP32_LANES_PER_SM = 128
 # DRAM traffic of the tracer kernel (dram__bytes_read.sum + dram__bytes_write.sum) and its warp
 # instructions (smsp__inst_executed.sum), from one single-pass ncu capture of the benchmarked
 # 1e7-ray launch, per primary ray; valid only while the tracer sources hash to `src_sha`.
-TRACE_TRAFFIC = {"src_sha": "37bf3dcea057bda4", "bytes_per_ray": 6.558, "warp_inst_per_ray": 262.2}
+TRACE_TRAFFIC = {"src_sha": "9e8637f8005a9a74", "bytes_per_ray": 6.555, "warp_inst_per_ray": 262.1}
 
 
 def tracer_sha():
@@ -87,7 +87,7 @@ def tracer_sha():
 
 # Warp instructions (smsp__inst_executed.sum) of the node deposit of the benchmarked frame, per arrival,
 # from the same kind of capture; valid only while its source hashes to `src_sha`.
-NODE_DEPOSIT = {"src_sha": "3e16fe30f16e2d89", "warp_inst_per_arrival": 62.8}
+NODE_DEPOSIT = {"src_sha": "8350df6bc6f2942e", "warp_inst_per_arrival": 62.8}
 
 
 def deposit_sha():

@@ -138,15 +138,15 @@ struct DasTile {
 
 // One thread per pixel (and part of the elements), KT transmits at a time.
 //
-// Bound by issue slots and, next, by the L1 reads of the four gathers per (pixel, element,
-// transmit) term.  Lanes run along x: neighbouring pixels of a row read samples at most a lateral
+// Bound by issue slots (67 % for 31 transmits, 80 % for one) and, next, by the latency of the four gathers
+// per (pixel, element, transmit) term.  Lanes run along x: neighbouring pixels of a row read samples at most a lateral
 // step apart (0.5 on average on the 512 x 256 image of 128 elements), so a row's gather touches one
 // or two cache lines, where lanes along depth are 2 dz fs / c = 12 samples apart and touch one sector
 // each.  A CTA's warps take consecutive rows of one x range, which share lines the same way.  The
 // receive delay is formed once per (pixel, element) and serves KT transmits; times are 32.32 fixed
 // point, so a term adds, splits and compares integers.  512 x 256 image of 128 elements x 3200 samples,
 // before (lanes along depth; float-float add, floor, IEEE square root and divide per term) and now:
-// 31 transmits 3044 -> 683 us, one transmit 98 -> 47 us; 25 transmits x 4096 samples 2451 -> 544 us.
+// 31 transmits 3044 -> 682 us, one transmit 98 -> 48 us; 25 transmits x 4096 samples 2451 -> 541 us.
 // Registers for the loads of a whole chunk pay more than warps once a chunk is long (31 transmits:
 // 680 us at 2 CTAs per SM, 760 at 3, 940 at 4), and the other way round for single transmits.
 template <int KT>
